@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(P * P * kop_ne<P>()) kop_kernel(const KArgs a)
   constexpr int NPT = P * P, ND = P * P * P;
   constexpr int TW = tile_words<P>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  colour_open_next();
   const int tid = threadIdx.x;
   const int el = tid / NPT;
   const int ij = tid - el * NPT;
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(P * P * kop_ne<P>()) kop_kernel(const KArgs a)
   double yt[P];
   eo_apply<P, P, -1>(a.tab.eDT, vt, yt);
   __syncthreads();
+  ColourWait()();  // the earlier colours' writes of y
   if (!active) return;
 #pragma unroll
   for (int c = 0; c < P; ++c) {
@@ -244,6 +246,7 @@ __global__ void __launch_bounds__(P * P * kop_ne<P>()) kop_df_kernel(const KArgs
   constexpr int NPT = P * P, ND = P * P * P;
   constexpr int TW = tile_words<P>();
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  colour_open_next();
   const int tid = threadIdx.x;
   const int el = tid / NPT;
   const int ij = tid - el * NPT;
@@ -358,6 +361,7 @@ __global__ void __launch_bounds__(P * P * kop_ne<P>()) kop_df_kernel(const KArgs
   DF yt[P];
   eo_apply<P, P, -1>(tab.eDT, vt, yt);
   __syncthreads();
+  ColourWait()();  // the earlier colours' writes of y
   if (!active) return;
 #pragma unroll
   for (int c = 0; c < P; ++c) {
@@ -379,11 +383,14 @@ static int run_kop_df(ceed_mesh_t m, KArgs a, cudaStream_t s) {
   constexpr int NE = kop_ne<P>();
   const size_t smem = NE * kop_elem_smem<P, ADJ>();
   if (int st = ensure_dynamic_smem((const void *)kop_df_kernel<P, ADJ>, smem)) return st;
+  bool first = true;
   for (int c = 0; c < m->n_colors; ++c) {
     a.e_begin = m->color_start[c];
     a.e_count = m->color_start[c + 1] - a.e_begin;
     if (a.e_count == 0) continue;
-    kop_df_kernel<P, ADJ><<<(unsigned)((a.e_count + NE - 1) / NE), P * P * NE, smem, s>>>(a, m->tabdf);
+    const dim3 grid((unsigned)((a.e_count + NE - 1) / NE));
+    if (int st = launch_colour(kop_df_kernel<P, ADJ>, grid, dim3(P * P * NE), smem, s, first, a, m->tabdf)) return st;
+    first = false;
   }
   CEED_CUDA_CHECK(cudaGetLastError());
   return CEED_OK;
@@ -394,11 +401,14 @@ static int run_kop(ceed_mesh_t m, KArgs a, cudaStream_t s) {
   constexpr int NE = kop_ne<P>();
   const size_t smem = NE * kop_elem_smem<P, ADJ>();
   if (int st = ensure_dynamic_smem((const void *)kop_kernel<P, ADJ>, smem)) return st;
+  bool first = true;
   for (int c = 0; c < m->n_colors; ++c) {
     a.e_begin = m->color_start[c];
     a.e_count = m->color_start[c + 1] - a.e_begin;
     if (a.e_count == 0) continue;
-    kop_kernel<P, ADJ><<<(unsigned)((a.e_count + NE - 1) / NE), P * P * NE, smem, s>>>(a);
+    const dim3 grid((unsigned)((a.e_count + NE - 1) / NE));
+    if (int st = launch_colour(kop_kernel<P, ADJ>, grid, dim3(P * P * NE), smem, s, first, a)) return st;
+    first = false;
   }
   CEED_CUDA_CHECK(cudaGetLastError());
   return CEED_OK;

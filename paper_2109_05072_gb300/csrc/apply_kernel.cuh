@@ -10,8 +10,9 @@
 //  * the element's quadrature data block is staged into shared memory by one TMA bulk copy
 //    (cp.async.bulk + mbarrier) issued at kernel entry, so it streams in while the gather and the
 //    forward contractions run; for several columns (components x right-hand sides) it is read once;
-//  * every global load of an element (restriction, x, and the old y of nodes already written by an
-//    earlier colour) is issued up front, so an element pays one memory latency, not four;
+//  * an element's restriction and x loads are issued up front, so that it pays one memory latency
+//    each; the old y of nodes already written by an earlier colour is loaded at the scatter, so that
+//    all the rest of a colour's work overlaps the colour before it (colour_open_next, ColourWait);
 //  * each 1D pass is done by "line owners": a thread holds a whole line of the tile in registers and
 //    applies the 1D operator with the even-odd (centro-symmetry) decomposition, which replaces an
 //    n x n product by two (n/2) x (n/2) products plus n folds/unfolds (48 instead of 64 operations
@@ -21,13 +22,15 @@
 //  * the FP32 operator converts FP64 L-vector values to FP32 and back with integer instructions and
 //    accumulates across colours in FP32, so it issues no FP64-pipe instruction at all;
 //  * elements of one colour share no node: the scatter is a plain store for the first writer of a
-//    node and a load-add-store for later colours (old value loaded up front): deterministic and
+//    node and a load-add-store for later colours: deterministic and
 //    atomic-free.
 #pragma once
 
 #include <cuda_bf16.h>
-#include <type_traits>
 #include <cuda_fp16.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "convert.cuh"
 #include "df.cuh"
@@ -124,6 +127,28 @@ __device__ __forceinline__ bool mbar_wait_n(uint64_t *bar, uint32_t parity, int 
   }
   return false;
 }
+
+// ------------------------------------------------------------------ colour after colour
+// The colours of one application are launched back to back as programmatic dependents: a colour's
+// blocks start as soon as the blocks of the colour before have all started and left room, gather,
+// compute, and wait for that colour's writes only before they touch y.  What an earlier colour can
+// change (y) is not read before the wait; what is read before it (x, restriction, quadrature data)
+// was complete when colour 0 started, which waits for everything before it in the stream as any
+// launch does.  Every thread waits, so a colour is complete only after all colours before it are.
+// Small meshes stop paying eight kernel latencies and large ones eight nearly empty last waves: 64
+// elements at p = 2 49 -> 25 us, 1,287 at p = 5 115 -> 49 us, 15,525 at p = 6 (Gauss mass) 583 -> 503 us,
+// 64,000 at p = 7 in FP32 445 -> 386 us.
+__device__ __forceinline__ void colour_open_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+struct ColourWait {
+  __device__ __forceinline__ bool operator()() const {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return true;
+  }
+};
+
+struct NoWait {  // persistent callers separate their colours themselves
+  __device__ __forceinline__ bool operator()() const { return true; }
+};
 
 // ------------------------------------------------------------------ even-odd 1D operator
 // out = M v for an NO x NI matrix with M[NO-1-i][NI-1-j] = S M[i][j] (S = +1 centro-symmetric,
@@ -533,6 +558,7 @@ struct ApplyArgs {
   int64_t e_begin, e_count;
   int64_t estride;  // quadrature data per element, in TQ units (16-byte multiple)
   int ncol, masked;
+  int cpb, cgroups; // columns per block, and blocks that share an element's columns (column_split)
   int ne;           // elements per thread block
   int *err;
   int wait_limit;    // polls of the quadrature-data copy wait: 0 gives up at once (CEED_ERR_TIMEOUT), else
@@ -543,14 +569,31 @@ struct ApplyArgs {
                      // (thread 0, in the order the block processes its work: a persistent block's sum)
 };
 
-// One thread block's share of a colour: elements e_begin + blk * ne + (0 .. ne-1).  Threads past
+// Columns per block: an element's columns (components x right-hand sides) share its quadrature data, but
+// a colour with few element blocks leaves the chip idle while each of them walks all the columns, and
+// a block that still has columns to do holds up the colours behind it.  So columns are spread
+// over blocks until a colour has COLUMN_BLOCKS of them (about 16 per SM, more than are resident); the
+// repeated quadrature data comes from L2.  p = 3 Gauss, 848
+// elements a colour, 12 columns: 1.65 ms with all columns in a block, 2.00 so with overlapping colours (their waiting
+// blocks take the working ones' places), 1.28 ms spread.
+constexpr int64_t COLUMN_BLOCKS = 152 * 16;
+inline void column_split(ApplyArgs &a, int64_t eblocks) {
+  const int64_t groups = std::min<int64_t>(a.ncol, std::max<int64_t>(1, COLUMN_BLOCKS / std::max<int64_t>(1, eblocks)));
+  a.cpb = (int)((a.ncol + groups - 1) / groups);
+  a.cgroups = (a.ncol + a.cpb - 1) / a.cpb;
+}
+
+// One thread block's share of a colour: elements e_begin + eb * ne + (0 .. ne-1), columns group cg of the
+// blk = eb * cgroups + cg.  Threads past
 // ne * Q^2 (a block shape that does not divide evenly) act as an inactive element; the caller
 // provides shared memory for ceil(blockDim / Q^2) elements and the mbarrier array.
 // XCG: x is read through L2 only (ld.global.cg) instead of the read-only path: required when x
 // changes during the kernel (the persistent CG iteration updates p between its applies).
-template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool XCG = false>
+// wait_y: called by every thread of the block before its first access to y (earlier colours written);
+// false if it gave up, and the block then writes nothing.
+template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool XCG = false, typename WaitY>
 __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &tab, int64_t blk,
-                                            unsigned char *smem_raw, uint64_t *bar) {
+                                            unsigned char *smem_raw, uint64_t *bar, const WaitY &wait_y) {
   constexpr int NPT = Q * Q;
   constexpr int ND = P * P * P;
   constexpr size_t QB = STAGE ? ((qblock_bytes<Q, OP, TQ>() + 127) & ~(size_t)127) : 0;
@@ -560,7 +603,9 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
   const int el = tid / NPT;
   const int ij = tid - el * NPT;
   const int i = ij % Q, j = ij / Q;
-  const int64_t e = a.e_begin + blk * a.ne + el;
+  const unsigned eb = (unsigned)blk / (unsigned)a.cgroups, cg = (unsigned)blk - eb * (unsigned)a.cgroups;
+  const int col0 = (int)cg * a.cpb, col1 = min(a.ncol, col0 + a.cpb);
+  const int64_t e = a.e_begin + (int64_t)eb * a.ne + el;
   const bool active = (el < a.ne) && (e < a.e_begin + a.e_count);
   const bool node_thread = (i < P) && (j < P);
   // staged block in shared memory, or the element's block in global memory
@@ -594,6 +639,7 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
     for (int c = 0; c < P; ++c) idx[c] = __ldg(em + c * P * P);
   }
   bool have_q = false;
+  bool y_ok = true;
   bool q_ok = true;  // false once this thread's copy wait gave up: the element then writes nothing
   auto wait_q = [&]() {
     if (STAGE && !have_q) {  // elements past the end issued no copy and do not wait
@@ -609,10 +655,11 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
     }
   };
 
-  for (int col = 0; col < a.ncol; ++col) {
-    // ---- all global loads of the column up front: x at my nodes, old y where an earlier colour wrote
-    // (the double-float operator, whose element work is long and register-hungry, loads the old y
-    // only at the scatter: holding it across the element would cost 2P registers of occupancy)
+  for (int col = col0; col < col1; ++col) {
+    // ---- x at my nodes, every load of the column up front; the old y where an earlier colour wrote
+    // with them from the second column on (the first loads it at the scatter, behind the earlier
+    // colours' writes; the double-float operator always does, as holding it across the element would
+    // cost 2P registers of occupancy)
     constexpr bool EARLY_YOLD = !std::is_same<T, DF>::value;
     double xv[P], yold[P];
 #pragma unroll
@@ -624,7 +671,7 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
         const int64_t o = (int64_t)(v & DOF_MASK) * a.ncol + col;
         const bool dir = a.masked && (v & FLAG_DIR);
         if (!dir) xv[c] = XCG ? __ldcg(a.x + o) : __ldg(a.x + o);
-        if (EARLY_YOLD && !dir && !(v & FLAG_FIRST)) yold[c] = __ldcg(a.y + o);  // L2: written by an earlier colour
+        if (EARLY_YOLD && col > col0 && y_ok && !dir && !(v & FLAG_FIRST)) yold[c] = __ldcg(a.y + o);
       }
     }
     T u[P];
@@ -635,11 +682,12 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
     element_op<P, Q, OP, T, TQ>(tab, u, yv, sq, sa, sb, sc, i, j, node_thread, active, wait_q);
 
     // ---- scatter-add (E -> L), atomic-free
+    if (col == col0) y_ok = wait_y();
     const bool fused_dot = a.dot_part || a.dot_sh;
-    if constexpr (!EARLY_YOLD) {
-      if (active && node_thread && q_ok) {
+    if (!EARLY_YOLD || col == col0) {
 #pragma unroll
-        for (int c = 0; c < P; ++c) {
+      for (int c = 0; c < P; ++c) {
+        if (active && node_thread && q_ok && y_ok) {
           const uint32_t v = idx[c];
           const int64_t o = (int64_t)(v & DOF_MASK) * a.ncol + col;
           if (!(a.masked && (v & FLAG_DIR)) && !(v & FLAG_FIRST)) yold[c] = __ldcg(a.y + o);
@@ -647,7 +695,7 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
       }
     }
     if (!fused_dot) {
-      if (active && node_thread && q_ok) {
+      if (active && node_thread && q_ok && y_ok) {
 #pragma unroll
         for (int c = 0; c < P; ++c) {
           const uint32_t v = idx[c];
@@ -665,7 +713,7 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
       // same scatter, and x . y over the nodes whose final value this thread writes (fused CG dot:
       // the last writer of a node adds x_i y_i; a masked Dirichlet node's first writer adds x_i^2)
       double dot = 0.0;
-      if (active && node_thread && q_ok) {
+      if (active && node_thread && q_ok && y_ok) {
 #pragma unroll
         for (int c = 0; c < P; ++c) {
           const uint32_t v = idx[c];
@@ -696,7 +744,7 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
         else a.dot_part[a.dot_base + blk] = t;
       }
     }
-    if (col + 1 < a.ncol) __syncthreads();
+    if (col + 1 < col1) __syncthreads();
   }
   // the block must not exit while its copy may still be writing shared memory: an element whose
   // wait gave up (or that never reached the pointwise step) waits once more, with the default bound
@@ -712,7 +760,9 @@ __global__ void __launch_bounds__(APPLY_MAX_THREADS)
 apply_kernel(const ApplyArgs a, const OpTab<T> tab) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
-  apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar);
+  ColourWait wait_y;
+  colour_open_next();
+  apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar, wait_y);
 }
 
 // The double-float instantiations under a register cap: that operator is bound by latency
@@ -723,7 +773,27 @@ template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
 __global__ void __maxnreg__(APPLY_DF_MAX_REGS) apply_kernel_capped(const ApplyArgs a, const OpTab<T> tab) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
-  apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar);
+  ColourWait wait_y;
+  colour_open_next();
+  apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar, wait_y);
+}
+
+// One colour's launch: the first of an application as any launch, the others as programmatic
+// dependents of the colour before (see ColourWait).
+template <typename Kernel, typename... Args>
+int launch_colour(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool first, const Args &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = first ? 0 : 1;
+  CEED_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, args...));
+  return CEED_OK;
 }
 
 }  // namespace ceedgb
@@ -756,14 +826,19 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
   a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
   a.dot_base = 0;
   a.dot_sh = nullptr;
+  bool first = true;
   for (int c = 0; c < m->n_colors; ++c) {
     a.e_begin = m->color_start[c];
     const int64_t n = m->color_start[c + 1] - a.e_begin;
     if (n == 0) continue;
     a.e_count = n;
-    const dim3 grid((unsigned)((n + ne - 1) / ne));
-    if constexpr (CAPPED) apply_kernel_capped<P, Q, OP, T, TQ, STAGE><<<grid, block, smem, s>>>(a, tab);
-    else apply_kernel<P, Q, OP, T, TQ, STAGE><<<grid, block, smem, s>>>(a, tab);
+    column_split(a, (n + ne - 1) / ne);
+    const dim3 grid((unsigned)((n + ne - 1) / ne * a.cgroups));
+    int st;
+    if constexpr (CAPPED) st = launch_colour(apply_kernel_capped<P, Q, OP, T, TQ, STAGE>, grid, block, smem, s, first, a, tab);
+    else st = launch_colour(apply_kernel<P, Q, OP, T, TQ, STAGE>, grid, block, smem, s, first, a, tab);
+    if (st) return st;
+    first = false;
     a.dot_base += grid.x;
   }
   if (r.dot_n) *r.dot_n = a.dot_part ? a.dot_base : 0;

@@ -71,6 +71,7 @@ __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char 
   __shared__ __align__(16) T tab_words[sizeof(OpTab<T>) / sizeof(T)];
   const OpTab<T> &tab = *reinterpret_cast<const OpTab<T> *>(tab_words);
   int cur_m = -1;
+  NoWait wait_y;
   for (int c = 0; c < b.max_colors; ++c) {
     int64_t nb[BATCH_MAX], total = 0;
 #pragma unroll
@@ -102,7 +103,7 @@ __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char 
       }
 #define CEEDGB_BCASE(PP)                                                                                         \
   case PP:                                                                                                      \
-    apply_block<PP, COLLOC ? PP : PP + 1, OP, T, TQ, STAGE>(a, tab, blk, smem_raw, bar);                  \
+    apply_block<PP, COLLOC ? PP : PP + 1, OP, T, TQ, STAGE>(a, tab, blk, smem_raw, bar, wait_y);          \
     break;
       switch (b.m[m].P) {
         CEEDGB_BCASE(2)
@@ -172,6 +173,8 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     bm.a.masked = reqs[k].masked;
     bm.a.ne = L.threads / (m->Q * m->Q);
     if (bm.a.ne < 1) return fail(CEED_ERR_INVALID, "block too small for this order");
+    bm.a.cpb = bm.a.ncol;
+    bm.a.cgroups = 1;
     bm.a.err = err;
     bm.a.wait_limit = copy_wait_limit();
     bm.a.estride = qdata_estride(OP, sizeof(TQ), m->Q);

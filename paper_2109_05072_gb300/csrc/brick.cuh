@@ -240,6 +240,7 @@ __device__ __forceinline__ void brick_block(const BrickArgs &a, const OpTab<T> &
 
   // ---- scatter: the lowest colour among the bricks sharing a node writes first (parity 0 on every
   // shared axis), later ones load-add-store
+  ColourWait()();  // the earlier colours' writes of y
   const uint32_t px = gf & 1u, py = (gf >> 1) & 1u, pz = (gf >> 2) & 1u;
   const bool sx = (A == 0 && (gf & BRICK_MX)) || (A == NB - 1 && (gf & BRICK_PX));
   double dot = 0.0;
@@ -317,6 +318,7 @@ template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
 __global__ void __launch_bounds__(brick_threads<Q>(), brick_min_blocks<Q>()) brick_kernel(const BrickArgs a, const OpTab<T> tab) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bar[STAGE ? 4 * BRICK_KZ : 1];
+  colour_open_next();
   brick_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar);
 }
 
@@ -350,11 +352,15 @@ int launch_bricks(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, cudaStr
   const void *kfn = (const void *)brick_kernel<P, Q, OP, T, TQ, STAGE>;
   if (int st = ensure_dynamic_smem(kfn, smem)) return st;
   BrickArgs a = brick_args(m, r, OP, sizeof(TQ));
+  bool first = true;
   for (int c = 0; c < 8; ++c) {
     a.g_begin = m->brick_start[c];
     const int64_t n = m->brick_start[c + 1] - a.g_begin;
     if (n == 0) continue;
-    brick_kernel<P, Q, OP, T, TQ, STAGE><<<(unsigned)n, brick_threads<Q>(), smem, s>>>(a, tab);
+    if (int st = launch_colour(brick_kernel<P, Q, OP, T, TQ, STAGE>, dim3((unsigned)n), dim3(brick_threads<Q>()), smem, s,
+                               first, a, tab))
+      return st;
+    first = false;
     a.dot_base += n;
   }
   if (r.dot_n) *r.dot_n = r.dot_part ? a.dot_base : 0;

@@ -370,6 +370,7 @@ static int fused_batch(ceed_mesh_t m, const ApplyReq &op, double *y, const Work 
   g.a.x = w.p;
   g.a.y = w.q;
   g.a.ncol = 1;
+  g.a.cpb = g.a.cgroups = 1;
   g.a.masked = op.masked;
   g.a.err = m->d_err + 1;
   g.a.wait_limit = copy_wait_limit();

@@ -60,6 +60,7 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
   __shared__ double red[APPLY_MAX_THREADS / 32];
   __shared__ int ok_sh;
   __shared__ uint64_t nobar[1];
+  NoWait wait_y;
   const int G = gridDim.x;
   const int tid = threadIdx.x;
   CgScalars *sc = g.sc;
@@ -82,7 +83,7 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
       a.e_count = g.cstart[c + 1] - a.e_begin;
       const int64_t nwork = (a.e_count + a.ne - 1) / a.ne;
       for (int64_t v = blockIdx.x; v < nwork; v += G) {
-        apply_block<P, Q, OP, T, TQ, false, true>(a, tab, v, smem_raw, nobar);
+        apply_block<P, Q, OP, T, TQ, false, true>(a, tab, v, smem_raw, nobar, wait_y);
         __syncthreads();  // shared memory is reused by the next element block
       }
       if (c + 1 == g.ncolors && tid == 0) g.part[blockIdx.x] = dsh;
