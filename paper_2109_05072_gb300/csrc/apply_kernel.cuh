@@ -146,10 +146,6 @@ struct ColourWait {
   }
 };
 
-struct NoWait {  // persistent callers separate their colours themselves
-  __device__ __forceinline__ bool operator()() const { return true; }
-};
-
 // ------------------------------------------------------------------ even-odd 1D operator
 // out = M v for an NO x NI matrix with M[NO-1-i][NI-1-j] = S M[i][j] (S = +1 centro-symmetric,
 // S = -1 centro-antisymmetric).  With e_j = v_j + v_{NI-1-j}, o_j = v_j - v_{NI-1-j} (j < NI/2):

@@ -1,8 +1,8 @@
 // Batched apply: several independent meshes (different polynomial orders allowed) in ONE persistent
-// launch.  Each thread block loops over the colours; within a colour it takes every G-th block of
-// work across all meshes (G = blocks in the grid), and a grid-wide barrier separates colours so that
-// the atomic-free scatter stays race-free.  The grid is sized to what is co-resident on the GPU;
-// the barrier's wait is bounded (a timeout is recorded instead of hanging).
+// launch.  The blocks of a persistent grid take pieces of work (element blocks) colour by colour over
+// all meshes; a piece touches y once its mesh's previous colour is in memory (ColourOrder), so that the
+// atomic-free scatter stays race-free.  The grid is sized to what is co-resident on the GPU; the wait
+// is bounded (a timeout is recorded instead of hanging).
 #pragma once
 
 #include <algorithm>
@@ -11,9 +11,6 @@
 #include "apply_kernel.cuh"
 
 namespace ceedgb {
-
-constexpr int BATCH_MAX = 4;
-constexpr int BATCH_MAX_COLORS = 16;
 
 struct BatchMesh {
   ApplyArgs a;                              // e_begin / e_count set per colour inside the kernel
@@ -24,9 +21,9 @@ struct BatchMesh {
 template <typename T>
 struct BatchArgs {
   int n, max_colors;
-  unsigned *sync;                           // [0] arrivals, [1] generation
+  unsigned *sync;                           // [BATCH_SYNC_WORDS], zero before a launch and after it
   int *err;
-  long long grid_wait;                      // polls of the grid barrier before it gives up
+  long long grid_wait;                      // polls of a wait between colours before it gives up
   BatchMesh m[BATCH_MAX];
   OpTab<T> tab[BATCH_MAX];
 };
@@ -62,6 +59,57 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, int *err, long long
   return *ok_sh != 0;
 }
 
+// Pieces of work (element blocks times column groups) of mesh m's colour c.
+template <typename T>
+__device__ __forceinline__ int64_t pieces(const BatchArgs<T> &b, int c, int m) {
+  if (c >= b.m[m].ncolors) return 0;
+  const ApplyArgs &a = b.m[m].a;
+  return (b.m[m].cstart[c + 1] - b.m[m].cstart[c] + a.ne - 1) / a.ne * a.cgroups;
+}
+
+// Order between the colours of a persistent apply without a grid barrier.  done[c] counts the pieces
+// of work (element blocks) of colour c that are in memory; a piece of colour c touches y once
+// done[c - 1] has reached its total -- every piece of colour c - 1 waited for colour c - 2, so all
+// earlier colours are then in memory.  Blocks take pieces in colour order, so the earliest unfinished
+// piece never waits, and all that a piece does before its scatter (gather, contractions) overlaps the
+// colour before.  The wait is bounded like the grid barrier's.
+struct ColourOrder {
+  const unsigned *prev;   // counter of the colour before; null: nothing to wait for
+  unsigned target;
+  long long limit;
+  int *err;
+  int *ok_sh;             // shared word: thread 0's verdict for the block
+  __device__ __forceinline__ bool operator()() const {
+    if (!prev) return true;
+    if (threadIdx.x == 0) {
+      int ok = 1;
+      const volatile unsigned *v = prev;
+      long long it = 0;
+      while (*v < target) {
+        if (++it > limit) {
+          ok = 0;
+          *err = CEED_ERR_TIMEOUT;
+          break;
+        }
+        __nanosleep(20);
+      }
+      __threadfence();
+      *ok_sh = ok;
+    }
+    __syncthreads();
+    return *ok_sh != 0;
+  }
+};
+
+// The block's piece of work is done (its writes included): called by every thread.
+__device__ __forceinline__ void colour_done(unsigned *done) {
+  __syncthreads();  // also frees shared memory for the next piece
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(done, 1u);
+  }
+}
+
 template <int OP, typename T, typename TQ, bool STAGE, bool COLLOC>
 __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char *smem_raw) {
   __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
@@ -70,62 +118,74 @@ __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char 
   // (indexing the parameter block by a run-time mesh slot would cost registers in every pass)
   __shared__ __align__(16) T tab_words[sizeof(OpTab<T>) / sizeof(T)];
   const OpTab<T> &tab = *reinterpret_cast<const OpTab<T> *>(tab_words);
+  __shared__ int64_t next_sh;
   int cur_m = -1;
-  NoWait wait_y;
-  for (int c = 0; c < b.max_colors; ++c) {
-    int64_t nb[BATCH_MAX], total = 0;
-#pragma unroll
-    for (int m = 0; m < BATCH_MAX; ++m) {
-      nb[m] = 0;
-      if (m < b.n && c < b.m[m].ncolors) {
-        const int64_t cnt = b.m[m].cstart[c + 1] - b.m[m].cstart[c];
-        nb[m] = (cnt + b.m[m].a.ne - 1) / b.m[m].a.ne;
-      }
-      total += nb[m];
+  int c = 0, m = 0;
+  int64_t base = 0;       // pieces before those of (colour c, mesh m)
+  int64_t cnt = pieces(b, 0, 0);
+  // pieces are numbered colour by colour, mesh by mesh, and handed out in that order: the orders'
+  // elements cost up to ten times one another, so a fixed share per block would leave blocks idle
+  if (threadIdx.x == 0) ok_sh = 1;
+  for (;;) {
+    if (threadIdx.x == 0) next_sh = atomicAdd(b.sync, 1u);
+    __syncthreads();
+    const int64_t v = next_sh;
+    if (v < base) {  // the counters went back under a running launch (the batch applied twice at once)
+      if (threadIdx.x == 0) *b.err = CEED_ERR_TIMEOUT;
+      return;
     }
-    for (int64_t v = blockIdx.x; v < total; v += gridDim.x) {
-      int m = 0;
-      int64_t base = 0;
-      while (v >= base + nb[m]) {
-        base += nb[m];
-        ++m;
+    while (v >= base + cnt) {
+      base += cnt;
+      if (++m == b.n) {
+        m = 0;
+        if (++c == b.max_colors) break;
       }
-      ApplyArgs a = b.m[m].a;
-      a.e_begin = b.m[m].cstart[c];
-      a.e_count = b.m[m].cstart[c + 1] - a.e_begin;
-      const int64_t blk = v - base;
-      if (m != cur_m) {
-        __syncthreads();
-        const T *src = reinterpret_cast<const T *>(&b.tab[m]);
-        for (int w = threadIdx.x; w < (int)(sizeof(OpTab<T>) / sizeof(T)); w += blockDim.x) tab_words[w] = src[w];
-        __syncthreads();
-        cur_m = m;
-      }
+      cnt = pieces(b, c, m);
+    }
+    if (c == b.max_colors) break;
+    ApplyArgs a = b.m[m].a;
+    a.e_begin = b.m[m].cstart[c];
+    a.e_count = b.m[m].cstart[c + 1] - a.e_begin;
+    unsigned *done = b.sync + 2 + m * BATCH_MAX_COLORS + c;
+    const ColourOrder wait_y{c ? done - 1 : nullptr, c ? (unsigned)pieces(b, c - 1, m) : 0u, b.grid_wait, b.err, &ok_sh};
+    const int64_t blk = v - base;
+    if (m != cur_m) {
+      const T *src = reinterpret_cast<const T *>(&b.tab[m]);
+      for (int w = threadIdx.x; w < (int)(sizeof(OpTab<T>) / sizeof(T)); w += blockDim.x) tab_words[w] = src[w];
+      __syncthreads();
+      cur_m = m;
+    }
 #define CEEDGB_BCASE(PP)                                                                                         \
   case PP:                                                                                                      \
     apply_block<PP, COLLOC ? PP : PP + 1, OP, T, TQ, STAGE>(a, tab, blk, smem_raw, bar, wait_y);          \
     break;
-      switch (b.m[m].P) {
-        CEEDGB_BCASE(2)
-        CEEDGB_BCASE(3)
-        CEEDGB_BCASE(4)
-        CEEDGB_BCASE(5)
-        CEEDGB_BCASE(6)
-        CEEDGB_BCASE(7)
-        CEEDGB_BCASE(8)
-        CEEDGB_BCASE(9)
-        default:
-          break;
-      }
-#undef CEEDGB_BCASE
-      __syncthreads();  // shared memory is reused by the next block of work
+    switch (b.m[m].P) {
+      CEEDGB_BCASE(2)
+      CEEDGB_BCASE(3)
+      CEEDGB_BCASE(4)
+      CEEDGB_BCASE(5)
+      CEEDGB_BCASE(6)
+      CEEDGB_BCASE(7)
+      CEEDGB_BCASE(8)
+      CEEDGB_BCASE(9)
+      default:
+        break;
     }
-    if (c + 1 < b.max_colors && !grid_barrier(b.sync, b.err, b.grid_wait, &ok_sh)) return;
+#undef CEEDGB_BCASE
+    if (!ok_sh) return;  // gave up: the later pieces' waits run out too; the host resets the counters
+    colour_done(done);
+  }
+  // the last block to leave readies the counters for the next launch (no block waits any more)
+  if (threadIdx.x == 0) {
+    if (atomicAdd(b.sync + 1, 1u) + 1u == gridDim.x) {
+      for (int w = 0; w < BATCH_SYNC_WORDS; ++w) b.sync[w] = 0u;
+      __threadfence();
+    }
   }
 }
 
 template <int OP, typename T, typename TQ, bool STAGE, bool COLLOC>
-__global__ void __launch_bounds__(APPLY_MAX_THREADS) batch_kernel(const BatchArgs<T> b) {
+__global__ void __launch_bounds__(APPLY_MAX_THREADS, std::is_same<T, DF>::value ? 1 : 2) batch_kernel(const BatchArgs<T> b) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   batch_body<OP, T, TQ, STAGE, COLLOC>(b, smem_raw);
 }
@@ -163,8 +223,9 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     BatchMesh &bm = b.m[k];
     bm.P = m->P;
     bm.Q = m->Q;
-    bm.ncolors = m->n_colors;
-    for (int c = 0; c <= m->n_colors; ++c) bm.cstart[c] = m->color_start[c];
+    bm.ncolors = 0;  // colours that hold elements (each waits for the one before)
+    for (int c = 0; c < m->n_colors; ++c)
+      if (m->color_start[c + 1] > m->color_start[c]) bm.cstart[++bm.ncolors] = m->color_start[c + 1];
     bm.a.emap = m->d_emap;
     bm.a.qdata = reqs[k].qdata;
     bm.a.x = reqs[k].x;
@@ -173,8 +234,7 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     bm.a.masked = reqs[k].masked;
     bm.a.ne = L.threads / (m->Q * m->Q);
     if (bm.a.ne < 1) return fail(CEED_ERR_INVALID, "block too small for this order");
-    bm.a.cpb = bm.a.ncol;
-    bm.a.cgroups = 1;
+    column_split(bm.a, (meshes[k]->E / std::max(1, bm.ncolors) + bm.a.ne - 1) / bm.a.ne);
     bm.a.err = err;
     bm.a.wait_limit = copy_wait_limit();
     bm.a.estride = qdata_estride(OP, sizeof(TQ), m->Q);
@@ -182,7 +242,7 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     bm.a.dot_base = 0;
     bm.a.dot_sh = nullptr;
     b.tab[k] = *tabs[k];
-    b.max_colors = std::max(b.max_colors, m->n_colors);
+    b.max_colors = std::max(b.max_colors, bm.ncolors);
     const size_t sm = L.stage ? batch_smem_for<OP, T, TQ, true>(m->P, m->Q, L.threads)
                               : batch_smem_for<OP, T, TQ, false>(m->P, m->Q, L.threads);
     smem = std::max(smem, sm);

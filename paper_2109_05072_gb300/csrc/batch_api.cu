@@ -100,10 +100,12 @@ extern "C" int ceed_batch_create(int n, const ceed_mesh_t *meshes, const void *c
     r.ncol = meshes[k]->ncomp * nrhs;
     r.masked = 0;
   }
-  cudaError_t e = cudaMalloc(&b->d_sync, 4 * sizeof(unsigned));
+  cudaError_t e = cudaMalloc(&b->d_sync, BATCH_SYNC_WORDS * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&b->d_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(b->d_sync, 0, 4 * sizeof(unsigned));
+  if (e == cudaSuccess) e = cudaMemset(b->d_sync, 0, BATCH_SYNC_WORDS * sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, sizeof(int));
+  // the memsets may still wait behind the default stream's work, which build_graph's stream does not
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
   if (e != cudaSuccess) {
     cudaFree(b->d_sync);
     cudaFree(b->d_err);
@@ -136,8 +138,8 @@ extern "C" int ceed_batch_status(ceed_batch_t b, void *stream) {
   int err = 0;
   CEED_CUDA_CHECK(cudaMemcpyAsync(&err, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, s));
   CEED_CUDA_CHECK(cudaStreamSynchronize(s));
-  if (err) {  // a bounded wait gave up: reset the barrier state for the next launch
-    CEED_CUDA_CHECK(cudaMemsetAsync(b->d_sync, 0, 4 * sizeof(unsigned), s));
+  if (err) {  // a bounded wait gave up: reset the counters for the next launch
+    CEED_CUDA_CHECK(cudaMemsetAsync(b->d_sync, 0, BATCH_SYNC_WORDS * sizeof(unsigned), s));
     CEED_CUDA_CHECK(cudaMemsetAsync(b->d_err, 0, sizeof(int), s));
     CEED_CUDA_CHECK(cudaStreamSynchronize(s));
     return fail(CEED_ERR_TIMEOUT, "a batched launch hit its grid-barrier or copy time limit");

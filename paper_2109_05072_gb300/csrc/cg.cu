@@ -276,7 +276,7 @@ struct Work {
   double *r_old;    // flexible CG: residual of the previous iteration
   double *pq_part;  // per-block partial sums of p . q written by the fused apply
   double *fpart;    // fused iteration: per-block partials [3][CGF_MAX_GRID]
-  unsigned *fsync;  // fused iteration: grid barrier state
+  unsigned *fsync;  // fused iteration: grid barrier state, finished work per colour
   Scalars *sc;
 };
 
@@ -302,7 +302,7 @@ static size_t layout(int64_t n, int64_t n_elem, bool mixed, char *base, Work *w)
   t.part1 = (double *)take(RED_MAX_BLOCKS * sizeof(double));
   t.part2 = (double *)take(RED_MAX_BLOCKS * sizeof(double));
   t.fpart = (double *)take(3 * CGF_MAX_GRID * sizeof(double));
-  t.fsync = (unsigned *)take(4 * sizeof(unsigned));
+  t.fsync = (unsigned *)take(CGF_SYNC_WORDS * sizeof(unsigned));
   t.sc = (Scalars *)take(sizeof(Scalars));
   if (w) *w = t;
   return off;
@@ -375,8 +375,8 @@ static int fused_batch(ceed_mesh_t m, const ApplyReq &op, double *y, const Work 
   g.a.err = m->d_err + 1;
   g.a.wait_limit = copy_wait_limit();
   g.a.estride = qdata_estride(qop, prec_size(op.prec), m->Q);
-  for (int c = 0; c <= m->n_colors; ++c) g.cstart[c] = m->color_start[c];
-  g.ncolors = m->n_colors;
+  for (int c = 0; c < m->n_colors; ++c)  // colours that hold elements (each waits for the one before)
+    if (m->color_start[c + 1] > m->color_start[c]) g.cstart[++g.ncolors] = m->color_start[c + 1];
   g.x = y;
   g.r = w.r;
   g.p = w.p;
@@ -387,11 +387,12 @@ static int fused_batch(ceed_mesh_t m, const ApplyReq &op, double *y, const Work 
   g.part = w.fpart;
   g.sc = w.sc;
   g.sync = w.fsync;
+  g.done = w.fsync + 4;
   g.grid_wait = grid_wait_limit();
   g.iters = iters;
   g.fixed = fixed ? 1 : 0;
   if (((uintptr_t)op.qdata & 15) != 0) return fail(CEED_ERR_INVALID, "qdata must be 16-byte aligned");
-  CEED_CUDA_CHECK(cudaMemsetAsync(w.fsync, 0, 4 * sizeof(unsigned), s));  // barrier state (a timeout leaves it dirty)
+  CEED_CUDA_CHECK(cudaMemsetAsync(w.fsync, 0, CGF_SYNC_WORDS * sizeof(unsigned), s));  // counters (a timeout leaves them dirty)
   // elements per block: the apply variant chosen for this operator (autotuner or
   // ceed_set_apply_variant), else blocks of about 128 threads
   const ApplyChoice &tc = m->tuned[CEED_OP_DIFFUSION][op.prec];

@@ -4,9 +4,10 @@
 // preconditioner; Section 2.4: the Krylov updates are memory-bound streaming work; Section 3: fusing
 // the operator's steps into one kernel removes global temporaries and launch gaps).
 //
-// The grid is launched cooperatively with as many blocks as can be resident at once, so that grid
-// barriers (bounded waits, as in the batched kernel) can separate the colours of the atomic-free
-// scatter and the phases of the iteration.  Every reduction has a fixed order: each block adds its
+// The grid is launched cooperatively with as many blocks as can be resident at once, so that bounded
+// waits on other blocks can separate the colours of the atomic-free
+// scatter (ColourOrder: by counters of finished work) and the phases of the iteration (grid barriers).
+// Every reduction has a fixed order: each block adds its
 // share in a fixed sequence, and every block then sums the blocks' partials in block order itself,
 // so all blocks hold the same alpha and beta and take the same stopping decision without another
 // barrier.  Block 0 publishes the scalars for the host.  The update stores z = D^{-1} r for the p
@@ -29,6 +30,7 @@ struct CgFusedArgs {
   double *part;                              // [3][gridDim]: p.q, r.z, r.r partials per block
   CgScalars *sc;
   unsigned *sync;                            // grid barrier state
+  unsigned *done;                            // finished pieces of work per colour, zero at launch
   long long grid_wait;
   int iters;                                 // iterations this launch may run
   int fixed;                                 // 1: run them all (no tolerance stop)
@@ -60,7 +62,6 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
   __shared__ double red[APPLY_MAX_THREADS / 32];
   __shared__ int ok_sh;
   __shared__ uint64_t nobar[1];
-  NoWait wait_y;
   const int G = gridDim.x;
   const int tid = threadIdx.x;
   CgScalars *sc = g.sc;
@@ -78,17 +79,25 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
     __syncthreads();
     ApplyArgs a = g.a;
     a.dot_sh = &dsh;
+    // pieces of work (element blocks) numbered colour by colour, every G-th one here (a fixed share:
+    // dsh adds them in a fixed order); the counters run on from one iteration to the next
+    int64_t base = 0;
+    unsigned before = 0;  // pieces of the colour before
     for (int c = 0; c < g.ncolors; ++c) {
       a.e_begin = g.cstart[c];
       a.e_count = g.cstart[c + 1] - a.e_begin;
       const int64_t nwork = (a.e_count + a.ne - 1) / a.ne;
-      for (int64_t v = blockIdx.x; v < nwork; v += G) {
+      const ColourOrder wait_y{c ? g.done + c - 1 : nullptr, before * (unsigned)(it + 1), g.grid_wait, &sc->timeout, &ok_sh};
+      for (int64_t v = (blockIdx.x + G - base % G) % G; v < nwork; v += G) {
         apply_block<P, Q, OP, T, TQ, false, true>(a, tab, v, smem_raw, nobar, wait_y);
-        __syncthreads();  // shared memory is reused by the next element block
+        if (c && !ok_sh) return;
+        colour_done(g.done + c);
       }
-      if (c + 1 == g.ncolors && tid == 0) g.part[blockIdx.x] = dsh;
-      if (!grid_barrier(g.sync, &sc->timeout, g.grid_wait, &ok_sh)) return;
+      base += nwork;
+      before = (unsigned)nwork;
     }
+    if (tid == 0) g.part[blockIdx.x] = dsh;
+    if (!grid_barrier(g.sync, &sc->timeout, g.grid_wait, &ok_sh)) return;
     // ---- alpha = r.z / p.q (every block sums the same partials in the same order)
     const double pq = cgf_sum_partials(g.part, G, red);
     const double alpha = rz / pq;

@@ -112,6 +112,10 @@ struct ApplyChoice {
 }  // namespace ceedgb
 
 namespace ceedgb {
+constexpr int BATCH_MAX = 4;
+constexpr int BATCH_MAX_COLORS = 16;
+// counters of a batch: next piece of work, blocks that have left, finished pieces per (mesh, colour)
+constexpr int BATCH_SYNC_WORDS = 2 + BATCH_MAX * BATCH_MAX_COLORS;
 // Launch shape of the persistent batched apply.
 struct BatchLaunch {
   int threads;     // threads per block
