@@ -795,6 +795,7 @@ int launch_colour(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_
 }  // namespace ceedgb
 
 #include "brick.cuh"
+#include "fix_apply.cuh"
 
 namespace ceedgb {
 
@@ -842,6 +843,43 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
   return CEED_OK;
 }
 
+// The slice kernel: one element per block, one launch per colour.
+template <int P, int Q, int OP>
+int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaStream_t s) {
+  constexpr size_t smem = fix_smem<P, Q, OP>();
+  if (int st = ensure_dynamic_smem((const void *)fix_kernel<P, Q, OP>, smem)) return st;
+  FixArgs f;
+  f.tab = m->d_fix;
+  ApplyArgs &a = f.a;
+  a.emap = m->d_emap;
+  a.qdata = r.qdata;
+  a.x = r.x;
+  a.y = r.y;
+  a.ncol = r.ncol;
+  a.masked = r.masked;
+  a.ne = 1;
+  a.err = m->d_err + 1;
+  a.wait_limit = copy_wait_limit();
+  a.estride = qdata_estride(OP, sizeof(double), Q);
+  a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
+  a.dot_base = 0;
+  a.dot_sh = nullptr;
+  bool first = true;
+  for (int c = 0; c < m->n_colors; ++c) {
+    a.e_begin = m->color_start[c];
+    a.e_count = m->color_start[c + 1] - a.e_begin;
+    if (a.e_count == 0) continue;
+    column_split(a, a.e_count);
+    if (int st = launch_colour(fix_kernel<P, Q, OP>, dim3((unsigned)(a.e_count * a.cgroups)), dim3(32 * fix_warps<Q>()), smem, s, first, f, tab))
+      return st;
+    first = false;
+    a.dot_base += a.e_count;
+  }
+  if (r.dot_n) *r.dot_n = a.dot_part ? a.dot_base : 0;
+  CEED_CUDA_CHECK(cudaGetLastError());
+  return CEED_OK;
+}
+
 template <int P, int Q, int OP, typename T, typename TQ>
 int launch_colours(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, cudaStream_t s) {
   int ne = r.ne, stage = r.stage;
@@ -862,8 +900,12 @@ int launch_colours(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, cudaSt
     stage = 1;
   }
   if (ne > max_elems_per_block<Q>() || ne > APPLY_MAX_NE) return fail(CEED_ERR_INVALID, "elements per block too large");
+  if constexpr (fix_covers<P, Q, OP, T>()) {
+    return launch_fix<P, Q, OP>(m, tab, r, s);
+  } else {
   if (stage) return launch_variant<P, Q, OP, T, TQ, true>(m, tab, r, ne, s);
   return launch_variant<P, Q, OP, T, TQ, false>(m, tab, r, ne, s);
+  }
 }
 
 // Dispatch on (P, collocated?) for one (op, T, TQ).

@@ -15,6 +15,7 @@ namespace ceedgb {
 struct BatchMesh {
   ApplyArgs a;                              // e_begin / e_count set per colour inside the kernel
   int P, Q, ncolors;
+  const uint32_t *fix;                      // digit tables of the slice kernels, if the mesh has them
   int64_t cstart[BATCH_MAX_COLORS + 1];     // colour-sorted element ranges
 };
 
@@ -28,19 +29,25 @@ struct BatchArgs {
   OpTab<T> tab[BATCH_MAX];
 };
 
+#ifndef COLOUR_POLL_NS
+#define COLOUR_POLL_NS 64
+#endif
+#ifndef BARRIER_POLL_NS
+#define BARRIER_POLL_NS 64
+#endif
 // Bounded grid barrier (sense by generation counter).  Returns false on timeout.
 __device__ __forceinline__ bool grid_barrier(unsigned *sync, int *err, long long limit, int *ok_sh) {
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    volatile unsigned *vgen = sync + 1;
+    volatile unsigned *vgen = sync + SYNC_LINE;
     const unsigned gen = *vgen;
     __threadfence();
     const unsigned arrived = atomicAdd(sync, 1u) + 1u;
     if (arrived == gridDim.x) {
       atomicExch(sync, 0u);
       __threadfence();
-      atomicAdd(sync + 1, 1u);
+      atomicAdd(sync + SYNC_LINE, 1u);
     } else {
       long long it = 0;
       while (*vgen == gen) {
@@ -49,7 +56,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, int *err, long long
           *err = CEED_ERR_TIMEOUT;
           break;
         }
-        __nanosleep(100);
+        __nanosleep(BARRIER_POLL_NS);
       }
     }
     __threadfence();
@@ -57,6 +64,13 @@ __device__ __forceinline__ bool grid_barrier(unsigned *sync, int *err, long long
   }
   __syncthreads();
   return *ok_sh != 0;
+}
+
+// The 1D tables of the mesh being processed, copied from the parameter block to the start of shared memory
+// (indexing the parameter block by a run-time mesh slot would cost registers in every pass).
+template <typename T>
+constexpr size_t batch_tab_bytes() {
+  return (sizeof(OpTab<T>) + 127) & ~(size_t)127;
 }
 
 // Pieces of work (element blocks times column groups) of mesh m's colour c.
@@ -91,7 +105,7 @@ struct ColourOrder {
           *err = CEED_ERR_TIMEOUT;
           break;
         }
-        __nanosleep(20);
+        __nanosleep(COLOUR_POLL_NS);
       }
       __threadfence();
       *ok_sh = ok;
@@ -110,14 +124,21 @@ __device__ __forceinline__ void colour_done(unsigned *done) {
   }
 }
 
+// One piece of work of one order: a function of its own, so that the orders' register needs do not add up (inlined
+// together under the cap of 128 registers they spill 1.8 KB per thread; here 48 bytes at most).
+template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
+__device__ __noinline__ void batch_piece(const ApplyArgs &a, const uint32_t *fix, int64_t blk, const ColourOrder &wait_y) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
+  const OpTab<T> &tab = *reinterpret_cast<const OpTab<T> *>(smem_raw);
+  if constexpr (fix_covers<P, Q, OP, T>()) fix_any_block<P, Q, OP, false>(a, tab, fix, blk, smem_raw + batch_tab_bytes<T>(), wait_y);
+  else apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blk, smem_raw + batch_tab_bytes<T>(), bar, wait_y);
+}
+
 template <int OP, typename T, typename TQ, bool STAGE, bool COLLOC>
 __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char *smem_raw) {
-  __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
   __shared__ int ok_sh;
-  // the 1D tables of the mesh being processed, copied from the parameter block into shared memory
-  // (indexing the parameter block by a run-time mesh slot would cost registers in every pass)
-  __shared__ __align__(16) T tab_words[sizeof(OpTab<T>) / sizeof(T)];
-  const OpTab<T> &tab = *reinterpret_cast<const OpTab<T> *>(tab_words);
+  T *tab_words = (T *)smem_raw;
   __shared__ int64_t next_sh;
   int cur_m = -1;
   int c = 0, m = 0;
@@ -146,8 +167,8 @@ __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char 
     ApplyArgs a = b.m[m].a;
     a.e_begin = b.m[m].cstart[c];
     a.e_count = b.m[m].cstart[c + 1] - a.e_begin;
-    unsigned *done = b.sync + 2 + m * BATCH_MAX_COLORS + c;
-    const ColourOrder wait_y{c ? done - 1 : nullptr, c ? (unsigned)pieces(b, c - 1, m) : 0u, b.grid_wait, b.err, &ok_sh};
+    unsigned *done = b.sync + (2 + m * BATCH_MAX_COLORS + c) * SYNC_LINE;
+    const ColourOrder wait_y{c ? done - SYNC_LINE : nullptr, c ? (unsigned)pieces(b, c - 1, m) : 0u, b.grid_wait, b.err, &ok_sh};
     const int64_t blk = v - base;
     if (m != cur_m) {
       const T *src = reinterpret_cast<const T *>(&b.tab[m]);
@@ -155,9 +176,9 @@ __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char 
       __syncthreads();
       cur_m = m;
     }
-#define CEEDGB_BCASE(PP)                                                                                         \
-  case PP:                                                                                                      \
-    apply_block<PP, COLLOC ? PP : PP + 1, OP, T, TQ, STAGE>(a, tab, blk, smem_raw, bar, wait_y);          \
+#define CEEDGB_BCASE(PP)                                                                       \
+  case PP:                                                                                     \
+    batch_piece<PP, COLLOC ? PP : PP + 1, OP, T, TQ, STAGE>(a, b.m[m].fix, blk, wait_y);       \
     break;
     switch (b.m[m].P) {
       CEEDGB_BCASE(2)
@@ -176,12 +197,10 @@ __device__ __forceinline__ void batch_body(const BatchArgs<T> &b, unsigned char 
     colour_done(done);
   }
   // the last block to leave readies the counters for the next launch (no block waits any more)
-  if (threadIdx.x == 0) {
-    if (atomicAdd(b.sync + 1, 1u) + 1u == gridDim.x) {
-      for (int w = 0; w < BATCH_SYNC_WORDS; ++w) b.sync[w] = 0u;
-      __threadfence();
-    }
-  }
+  if (threadIdx.x == 0) ok_sh = atomicAdd(b.sync + SYNC_LINE, 1u) + 1u == gridDim.x;
+  __syncthreads();
+  if (ok_sh)
+    for (int w = threadIdx.x * SYNC_LINE; w < BATCH_SYNC_WORDS; w += blockDim.x * SYNC_LINE) b.sync[w] = 0u;
 }
 
 template <int OP, typename T, typename TQ, bool STAGE, bool COLLOC>
@@ -190,9 +209,28 @@ __global__ void __launch_bounds__(APPLY_MAX_THREADS, std::is_same<T, DF>::value 
   batch_body<OP, T, TQ, STAGE, COLLOC>(b, smem_raw);
 }
 
+// Threads of one element where the slice kernels run the mesh's operator, else 0.
+template <int OP, typename T>
+int batch_fix_threads(int P, int Q) {
+#define CEEDGB_S(PP)                                                                                   \
+  if (P == PP && Q == PP && fix_covers<PP, PP, OP, T>()) return 32 * fix_warps<PP>();                   \
+  if (P == PP && Q == PP + 1 && fix_covers<PP, PP + 1, OP, T>()) return 32 * fix_warps<PP + 1>();
+  CEEDGB_S(6) CEEDGB_S(7) CEEDGB_S(8)
+#undef CEEDGB_S
+  return 0;
+}
+
 // Shared memory per thread block for a mesh with P nodes / Q points when blocks have `threads` threads.
 template <int OP, typename T, typename TQ, bool STAGE>
 size_t batch_smem_for(int P, int Q, int threads) {
+  if (const int per = batch_fix_threads<OP, T>(P, Q)) {
+    size_t fb = 0;
+#define CEEDGB_S(PP) \
+  if (P == PP) fb = (Q == PP) ? fix_smem<PP, PP, OP>() : fix_smem<PP, PP + 1, OP>();
+    CEEDGB_S(6) CEEDGB_S(7) CEEDGB_S(8)
+#undef CEEDGB_S
+    return (size_t)((threads + per - 1) / per) * fb;
+  }
   const int slots = (threads + Q * Q - 1) / (Q * Q);
   size_t eb = 0;
 #define CEEDGB_S(PP)                                                                              \
@@ -232,7 +270,9 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     bm.a.y = reqs[k].y;
     bm.a.ncol = reqs[k].ncol;
     bm.a.masked = reqs[k].masked;
-    bm.a.ne = L.threads / (m->Q * m->Q);
+    const int fix_threads = batch_fix_threads<OP, T>(m->P, m->Q);
+    bm.fix = m->d_fix;
+    bm.a.ne = L.threads / (fix_threads ? fix_threads : m->Q * m->Q);
     if (bm.a.ne < 1) return fail(CEED_ERR_INVALID, "block too small for this order");
     column_split(bm.a, (meshes[k]->E / std::max(1, bm.ncolors) + bm.a.ne - 1) / bm.a.ne);
     bm.a.err = err;
@@ -245,7 +285,7 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     b.max_colors = std::max(b.max_colors, bm.ncolors);
     const size_t sm = L.stage ? batch_smem_for<OP, T, TQ, true>(m->P, m->Q, L.threads)
                               : batch_smem_for<OP, T, TQ, false>(m->P, m->Q, L.threads);
-    smem = std::max(smem, sm);
+    smem = std::max(smem, batch_tab_bytes<T>() + sm);
   }
   auto go = [&](auto kernel) -> int {
     CEED_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

@@ -382,12 +382,13 @@ static int fused_batch(ceed_mesh_t m, const ApplyReq &op, double *y, const Work 
   g.p = w.p;
   g.q = w.q;
   g.z = w.z;
+  g.fix = m->d_fix;
   g.dinv = w.dinv;
   g.n = n;
   g.part = w.fpart;
   g.sc = w.sc;
   g.sync = w.fsync;
-  g.done = w.fsync + 4;
+  g.done = w.fsync + 2 * SYNC_LINE;
   g.grid_wait = grid_wait_limit();
   g.iters = iters;
   g.fixed = fixed ? 1 : 0;

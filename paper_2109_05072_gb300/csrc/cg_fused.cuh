@@ -31,6 +31,7 @@ struct CgFusedArgs {
   CgScalars *sc;
   unsigned *sync;                            // grid barrier state
   unsigned *done;                            // finished pieces of work per colour, zero at launch
+  const uint32_t *fix;                       // digit tables (operators the slice kernel covers)
   long long grid_wait;
   int iters;                                 // iterations this launch may run
   int fixed;                                 // 1: run them all (no tolerance stop)
@@ -87,11 +88,12 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
       a.e_begin = g.cstart[c];
       a.e_count = g.cstart[c + 1] - a.e_begin;
       const int64_t nwork = (a.e_count + a.ne - 1) / a.ne;
-      const ColourOrder wait_y{c ? g.done + c - 1 : nullptr, before * (unsigned)(it + 1), g.grid_wait, &sc->timeout, &ok_sh};
+      const ColourOrder wait_y{c ? g.done + (c - 1) * SYNC_LINE : nullptr, before * (unsigned)(it + 1), g.grid_wait, &sc->timeout, &ok_sh};
       for (int64_t v = (blockIdx.x + G - base % G) % G; v < nwork; v += G) {
-        apply_block<P, Q, OP, T, TQ, false, true>(a, tab, v, smem_raw, nobar, wait_y);
+        if constexpr (fix_covers<P, Q, OP, T>()) fix_block<Q, true>(a, tab, g.fix, v, smem_raw, wait_y);
+        else apply_block<P, Q, OP, T, TQ, false, true>(a, tab, v, smem_raw, nobar, wait_y);
         if (c && !ok_sh) return;
-        colour_done(g.done + c);
+        colour_done(g.done + c * SYNC_LINE);
       }
       base += nwork;
       before = (unsigned)nwork;
@@ -215,9 +217,9 @@ __global__ void __maxnreg__(REGS) cg_fused_kernel(const CgFusedArgs g, const OpT
   cg_fused_body<P, Q, OP, T, TQ>(g, tab, smem_raw);
 }
 
-template <typename T>
+template <int P, int Q, int OP, typename T>
 constexpr int cgf_max_regs() {
-  return std::is_same<T, DF>::value ? APPLY_DF_MAX_REGS
+  return (std::is_same<T, DF>::value || fix_covers<P, Q, OP, T>()) ? APPLY_DF_MAX_REGS
          : std::is_same<T, float>::value ? CGF_F32_MAX_REGS
                                          : CGF_F64_MAX_REGS;
 }
@@ -227,12 +229,14 @@ constexpr int cgf_max_regs() {
 template <int P, int OP, typename T, typename TQ>
 int launch_cg_fused(const CgFusedArgs &gin, const OpTab<T> &tab, int ne, cudaStream_t s, unsigned *grid_out) {
   constexpr int Q = P;
-  constexpr int REGS = cgf_max_regs<T>();
+  constexpr int REGS = cgf_max_regs<P, Q, OP, T>();
   if (ne < 1 || ne > max_elems_per_block<Q>() || ne > APPLY_MAX_NE) return fail(CEED_ERR_INVALID, "bad elements per block");
-  const size_t smem = (size_t)ne * apply_elem_smem<P, Q, OP, T, TQ, false>();
+  constexpr bool FIX = fix_covers<P, Q, OP, T>();
+  if (FIX) ne = 1;
+  const size_t smem = FIX ? fix_smem<P, Q, OP>() : (size_t)ne * apply_elem_smem<P, Q, OP, T, TQ, false>();
   const void *kfn = (const void *)cg_fused_kernel<P, Q, OP, T, TQ, REGS>;
   if (int st = ensure_dynamic_smem(kfn, smem)) return st;
-  const int threads = Q * Q * ne;
+  const int threads = FIX ? 32 * fix_warps<Q>() : Q * Q * ne;
   int per_sm = 0, dev = 0, nsm = 0;
   CEED_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, threads, smem));
   CEED_CUDA_CHECK(cudaGetDevice(&dev));

@@ -8,7 +8,7 @@
 namespace ceedgb {
 
 constexpr int CGF_MAX_COLORS = 64;
-constexpr int CGF_SYNC_WORDS = 4 + CGF_MAX_COLORS;  // grid barrier (4 words), finished work per colour
+constexpr int CGF_SYNC_WORDS = (2 + CGF_MAX_COLORS) * SYNC_LINE;  // grid barrier (2 lines), finished work per colour
 constexpr int CGF_MAX_GRID = 8192;     // resident blocks of a fused launch (partials per reduction)
 
 struct CgFusedArgs;

@@ -95,6 +95,16 @@ struct CgScalars {
   int done, iters, nonfinite, timeout;  // timeout: a grid barrier of the fused iteration gave up
 };
 
+// Digit tables of the slice kernels (fixmma.cuh): eight words per lane and the scale.
+constexpr int FIX_DIGITS = 8;
+constexpr int FIX_TAB_WORDS = FIX_DIGITS * 32 + 32;
+constexpr int FIX_MIN_Q = 6, FIX_MAX_Q = 8;  // points per direction the slice kernel covers
+
+// A value's eight balanced base-256 digits as FP16 bit patterns, leading digit first: the integer nearest
+// to v 2^scale, which has to lie below 2^62 (mesh.cu).
+void fix_digits_host(long double v, int scale, uint16_t *out);
+int fix_scale_host(const long double *M, size_t n);  // largest scale that keeps every entry below 2^62
+
 struct QRule {
   double x[MAX_Q];
   double w[MAX_Q];
@@ -114,8 +124,10 @@ struct ApplyChoice {
 namespace ceedgb {
 constexpr int BATCH_MAX = 4;
 constexpr int BATCH_MAX_COLORS = 16;
-// counters of a batch: next piece of work, blocks that have left, finished pieces per (mesh, colour)
-constexpr int BATCH_SYNC_WORDS = 2 + BATCH_MAX * BATCH_MAX_COLORS;
+// counters of a batch, each on a 128-byte line of its own (waiting blocks read one while others are counted up): next piece
+// of work, blocks that have left, finished pieces per (mesh, colour)
+constexpr int SYNC_LINE = 32;
+constexpr int BATCH_SYNC_WORDS = (2 + BATCH_MAX * BATCH_MAX_COLORS) * SYNC_LINE;
 // Launch shape of the persistent batched apply.
 struct BatchLaunch {
   int threads;     // threads per block
@@ -135,6 +147,7 @@ struct ceed_mesh_s {
   double *d_vertices = nullptr;         // [E][8][3] colour-sorted
   double *d_coords = nullptr;           // [n_ldof][3] curved (isoparametric) node positions, or null
   int *d_err = nullptr;                 // device status word
+  uint32_t *d_fix = nullptr;            // [4][FIX_TAB_WORDS] digit tables of D, D^T, B, B^T (FIX_MIN_Q..FIX_MAX_Q points)
   bool has_dirichlet = false;
   ceedgb::OpTab<double> tab64;
   ceedgb::OpTab<float> tab32;

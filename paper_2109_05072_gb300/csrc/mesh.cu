@@ -9,6 +9,8 @@
 #include <new>
 #include <utility>
 
+#include <cuda_fp16.h>
+
 #include "internal.h"
 
 namespace ceedgb {
@@ -206,6 +208,55 @@ static void make_eo(const double *M, int NO, int NI, int S, EOMat<double> *d, EO
   for (size_t k = 0; k < sizeof(*d) / sizeof(double); ++k) dst[k] = (float)src[k];
 }
 
+int fix_scale_host(const long double *M, size_t n) {
+  long double big = 0;
+  for (size_t k = 0; k < n; ++k) big = std::max(big, std::fabs(M[k]));
+  int ex = 0;
+  std::frexp(big, &ex);  // big < 2^ex
+  return 62 - ex;
+}
+
+void fix_digits_host(long double v, int scale, uint16_t *out) {
+  int64_t r = std::llrint(std::ldexp(v, scale));
+  for (int j = FIX_DIGITS - 1; j >= 0; --j) {
+    const int dig = (int)(((r + 128) & 255) - 128);
+    r = (r - dig) / 256;
+    const __half h = __float2half_rn((float)dig);  // |digit| <= 128: exact
+    std::memcpy(&out[j], &h, 2);
+  }
+}
+
+// Digit table of an NO x NI matrix (both at most 8) for the slice kernels' B fragments.  The matrix is the one that
+// the even-odd blocks stand for (symmetric or antisymmetric to the last bit), so that both kinds of kernel apply
+// the same operator.  Word [j * 32 + lane]
+// holds digit j of M[g][2t] and M[g][2t + 1], g = lane / 4, t = lane % 4 (zero past the matrix); then the scale.
+static void fix_table(const EOMat<double> &eo, int NO, int NI, int S, uint32_t *out) {
+  long double M[MAX_Q * MAX_Q];
+  const int HO = NO / 2, HI = NI / 2;
+  for (int i = 0; i < HO; ++i)
+    for (int j = 0; j < NI; ++j) {
+      const long double E = j == HI && (NI & 1) ? eo.cmid[i] : eo.E[i * EO_H + std::min(j, NI - 1 - j)];
+      const long double O = j == HI && (NI & 1) ? 0.0 : eo.O[i * EO_H + std::min(j, NI - 1 - j)];
+      const long double v = j < NI - 1 - j ? E + O : E - O;
+      M[i * NI + j] = v;
+      M[(NO - 1 - i) * NI + NI - 1 - j] = S * v;
+    }
+  if (NO & 1)
+    for (int j = 0; j < NI; ++j)
+      M[HO * NI + j] = j == HI && (NI & 1) ? eo.cc : (j < HI ? 1 : S) * eo.rmid[std::min(j, NI - 1 - j)];
+  const int scale = fix_scale_host(M, (size_t)NO * NI);
+  for (int k = 0; k < FIX_TAB_WORDS; ++k) out[k] = 0;
+  out[FIX_DIGITS * 32] = (uint32_t)scale;
+  for (int lane = 0; lane < 32; ++lane)
+    for (int h = 0; h < 2; ++h) {
+      const int g = lane / 4, m = 2 * (lane % 4) + h;
+      if (g >= NO || m >= NI) continue;
+      uint16_t dig[FIX_DIGITS];
+      fix_digits_host(M[g * NI + m], scale, dig);
+      for (int j = 0; j < FIX_DIGITS; ++j) out[j * 32 + lane] |= (uint32_t)dig[j] << (16 * h);
+    }
+}
+
 static void build_tables(ceed_mesh_s *m) {
   double w_gll[MAX_P];
   gll_rule(m->P, m->gll_x, w_gll);
@@ -305,6 +356,7 @@ struct HostFree {
     cudaFree(m->d_vertices);
     cudaFree(m->d_coords);
     cudaFree(m->d_err);
+    cudaFree(m->d_fix);
     cudaFree(m->d_gbase);
     cudaFree(m->d_gelem);
     cudaFree(m->d_gflags);
@@ -572,6 +624,17 @@ extern "C" int ceed_setup_mesh(const ceed_mesh_desc *desc, ceed_mesh_t *out, voi
   CEED_CUDA_CHECK(cudaMemcpyAsync(m->d_perm, perm.data(), E * 4, cudaMemcpyHostToDevice, s));
   CEED_CUDA_CHECK(cudaMemcpyAsync(m->d_vertices, svert.data(), E * 24 * 8, cudaMemcpyHostToDevice, s));
   CEED_CUDA_CHECK(cudaMemsetAsync(m->d_err, 0, sizeof(int) * 4, s));
+  std::vector<uint32_t> fix;
+  if (m->Q >= FIX_MIN_Q && m->Q <= FIX_MAX_Q) {
+    const int P = m->P, Q = m->Q;
+    fix.resize(4 * FIX_TAB_WORDS);
+    fix_table(m->tab64.eD, Q, Q, -1, &fix[0]);
+    fix_table(m->tab64.eDT, Q, Q, -1, &fix[FIX_TAB_WORDS]);
+    fix_table(m->tab64.eB, Q, P, +1, &fix[2 * FIX_TAB_WORDS]);
+    fix_table(m->tab64.eBT, P, Q, +1, &fix[3 * FIX_TAB_WORDS]);
+    CEED_CUDA_CHECK(cudaMalloc(&m->d_fix, fix.size() * 4));
+    CEED_CUDA_CHECK(cudaMemcpyAsync(m->d_fix, fix.data(), fix.size() * 4, cudaMemcpyHostToDevice, s));
+  }
   if (desc->coords) {  // curved geometry: the handle keeps its own copy of the node positions
     CEED_CUDA_CHECK(cudaMalloc(&m->d_coords, nL * 3 * sizeof(double)));
     CEED_CUDA_CHECK(cudaMemcpyAsync(m->d_coords, desc->coords, nL * 3 * sizeof(double), cudaMemcpyDefault, s));
