@@ -23,6 +23,7 @@
 #include <cstring>
 #include <memory>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "geometry.cuh"
@@ -550,7 +551,11 @@ static int nt_apply_t(ceed_nt_t h, const NtChoice &c, const T *tab, const T *qd,
   T *Ye = reinterpret_cast<T *>(h->d_evec);
   int st;
   if (c.algo == CEED_NT_FUSED) {
-    st = launch_fused<T, D>(h, tab, qd, x, Ye, masked, s);
+    if (std::is_same<T, double>::value && nt_fix_supported(h->P))
+      st = nt_fix_apply(h, D == 1 ? CEED_OP_MASS : CEED_OP_DIFFUSION, reinterpret_cast<const double *>(qd), x,
+                        reinterpret_cast<double *>(Ye), masked, s);
+    else
+      st = launch_fused<T, D>(h, tab, qd, x, Ye, masked, s);
   } else if (c.algo == CEED_NT_TC) {
     if (sizeof(T) != 4) return fail(CEED_ERR_UNSUPPORTED, "tensor-core algorithm: F32 only");
     st = nt_tc_apply(h, D == 1 ? CEED_OP_MASS : CEED_OP_DIFFUSION, reinterpret_cast<const float *>(qd), x,
@@ -645,6 +650,8 @@ struct NtFree {
     cudaFree(h->d_s);
     cudaFree(h->d_tc_tab[0]);
     cudaFree(h->d_tc_tab[1]);
+    cudaFree(h->d_fix[0]);
+    cudaFree(h->d_fix[1]);
     delete h;
   }
 };
@@ -758,6 +765,8 @@ extern "C" int ceed_nt_setup(const ceed_nt_desc *desc, ceed_nt_t *out, void *str
   CEED_CUDA_CHECK(cudaMemcpyAsync(h->d_dir, dir.data(), (size_t)nL, cudaMemcpyHostToDevice, s));
   CEED_CUDA_CHECK(cudaMemcpyAsync(h->d_vert, desc->vertices, (size_t)E * 96, cudaMemcpyDeviceToDevice, s));
   CEED_CUDA_CHECK(cudaMemsetAsync(h->d_err, 0, sizeof(int), s));
+  if (nt_fix_supported(P))
+    if (int st = nt_fix_prepare(h.get(), tab64.data(), s)) return st;
   cublasStatus_t bs = cublasCreate(&h->blas);
   if (bs != CUBLAS_STATUS_SUCCESS) {
     h->blas = nullptr;
