@@ -146,6 +146,28 @@ struct ColourWait {
   }
 };
 
+// A mesh small enough for one thread-block cluster: all its colours in one launch.  Every block gathers and
+// computes its elements at once, then the colours take turns at y, a cluster barrier between them (y is
+// read and written through L2).
+constexpr int CLUSTER_BLOCKS = 8;
+constexpr int CLUSTER_COLORS = 16;
+struct ClusterOrder {
+  int ncolors;
+  int start[CLUSTER_COLORS + 1];   // colour-sorted element ranges
+  // f(true) in element e's turn, f(false) in the others
+  template <typename F>
+  __device__ __forceinline__ void in_turn(int64_t e, F f) const {
+#pragma unroll 1
+    for (int c = 0; c < ncolors; ++c) {
+      f(e >= start[c] && e < start[c + 1]);
+      if (c + 1 < ncolors) {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+      }
+    }
+  }
+};
+
 // ------------------------------------------------------------------ even-odd 1D operator
 // out = M v for an NO x NI matrix with M[NO-1-i][NI-1-j] = S M[i][j] (S = +1 centro-symmetric,
 // S = -1 centro-antisymmetric).  With e_j = v_j + v_{NI-1-j}, o_j = v_j - v_{NI-1-j} (j < NI/2):
@@ -678,7 +700,31 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
     element_op<P, Q, OP, T, TQ>(tab, u, yv, sq, sa, sb, sc, i, j, node_thread, active, wait_q);
 
     // ---- scatter-add (E -> L), atomic-free
-    if (col == col0) y_ok = wait_y();
+    if constexpr (std::is_same<WaitY, ClusterOrder>::value) {  // one column per block, no fused dot
+      wait_y.in_turn(e, [&](bool turn) {
+        if (!(turn && active && node_thread && q_ok)) return;
+        double yold[P];
+#pragma unroll
+        for (int c = 0; c < P; ++c) {
+          const uint32_t v = idx[c];
+          yold[c] = 0.0;
+          if (!(a.masked && (v & FLAG_DIR)) && !(v & FLAG_FIRST)) yold[c] = __ldcg(a.y + (int64_t)(v & DOF_MASK) * a.ncol + col);
+        }
+#pragma unroll
+        for (int c = 0; c < P; ++c) {
+          const uint32_t v = idx[c];
+          const int64_t o = (int64_t)(v & DOF_MASK) * a.ncol + col;
+          if (a.masked && (v & FLAG_DIR)) {
+            if (v & FLAG_FIRST) a.y[o] = a.x[o];
+          } else {
+            a.y[o] = (v & FLAG_FIRST) ? LVec<T>::out(yv[c]) : LVec<T>::add(yold[c], yv[c]);
+          }
+        }
+      });
+      continue;
+    } else if (col == col0) {
+      y_ok = wait_y();
+    }
     const bool fused_dot = a.dot_part || a.dot_sh;
     if (!EARLY_YOLD || col == col0) {
 #pragma unroll
@@ -799,6 +845,51 @@ int launch_colour(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_
 
 namespace ceedgb {
 
+template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
+__global__ void __launch_bounds__(APPLY_MAX_THREADS) apply_cluster_kernel(const ApplyArgs a, const OpTab<T> tab, const ClusterOrder order) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
+  apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar, order);
+}
+
+// Elements per block if the mesh's elements times the columns fit one cluster (at most max_ne elements a block), else 0.
+// The rule is the launch's own limit: up to there one launch beats eight overlapping ones (64 elements at p = 2: 13 to 16 us against
+// 24.8).
+inline int cluster_elems(ceed_mesh_t m, const ApplyReq &r, int max_ne) {
+  if (r.dot_part || r.ncol > CLUSTER_BLOCKS || m->n_colors > CLUSTER_COLORS) return 0;
+  const int64_t per_column = CLUSTER_BLOCKS / r.ncol, ne = (m->E + per_column - 1) / per_column;
+  return ne <= max_ne ? (int)ne : 0;
+}
+
+// Launch `kernel` as one cluster over all colours (a.ne elements and one column per block).
+template <typename Kernel, typename Args, typename Tab>
+int launch_cluster(ceed_mesh_t m, Kernel kernel, ApplyArgs &a, const Args &args, const Tab &tab, int threads, size_t smem, cudaStream_t s) {
+  ClusterOrder order;
+  order.ncolors = m->n_colors;
+  for (int c = 0; c <= m->n_colors; ++c) order.start[c] = (int)m->color_start[c];
+  a.e_begin = 0;
+  a.e_count = m->E;
+  a.cpb = 1;
+  a.cgroups = a.ncol;
+  // (+ 1024: the kernel's static shared memory counts against the default limit too)
+  if (int st = ensure_dynamic_smem((const void *)kernel, smem + 1024)) return st;
+  const unsigned grid = (unsigned)((m->E + a.ne - 1) / a.ne * a.ncol);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = grid;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  CEED_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, args, tab, order));
+  return CEED_OK;
+}
+
 // Launch one kernel per colour for a fixed (P, Q, op, T, TQ) and variant (elements per block, staging).
 template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
 int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne, cudaStream_t s) {
@@ -823,6 +914,12 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
   a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
   a.dot_base = 0;
   a.dot_sh = nullptr;
+  if (const int cne = cluster_elems(m, r, std::min(max_elems_per_block<Q>(), APPLY_MAX_NE))) {
+    a.ne = cne;
+    if (r.dot_n) *r.dot_n = 0;
+    return launch_cluster(m, apply_cluster_kernel<P, Q, OP, T, TQ, STAGE>, a, a, tab, Q * Q * cne,
+                          (size_t)cne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>(), s);
+  }
   bool first = true;
   for (int c = 0; c < m->n_colors; ++c) {
     a.e_begin = m->color_start[c];
@@ -864,6 +961,11 @@ int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaS
   a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
   a.dot_base = 0;
   a.dot_sh = nullptr;
+  if (const int cne = cluster_elems(m, r, APPLY_MAX_THREADS / (32 * fix_warps<Q>()))) {
+    a.ne = cne;
+    if (r.dot_n) *r.dot_n = 0;
+    return launch_cluster(m, fix_cluster_kernel<P, Q, OP>, a, f, tab, 32 * fix_warps<Q>() * cne, cne * fix_smem<P, Q, OP>(), s);
+  }
   bool first = true;
   for (int c = 0; c < m->n_colors; ++c) {
     a.e_begin = m->color_start[c];

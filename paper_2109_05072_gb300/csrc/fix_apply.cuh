@@ -68,6 +68,23 @@ __device__ __forceinline__ void fix_scatter(const ApplyArgs &a, const uint32_t (
   }
 }
 
+// fix_scatter in the element's turn; false if the wait for it gave up (nothing is then written).
+template <bool XCG, typename WaitY>
+__device__ __forceinline__ bool fix_turn(const ApplyArgs &a, const uint32_t (&idx)[4], const bool (&on)[4], const double (&r)[4],
+                                         int64_t e, int col, bool first_col, int64_t blk, const WaitY &wait_y) {
+  if constexpr (std::is_same<WaitY, ClusterOrder>::value) {
+    wait_y.in_turn(e, [&](bool turn) {
+      const bool now[4] = {turn && on[0], turn && on[1], turn && on[2], turn && on[3]};
+      fix_scatter<XCG>(a, idx, now, r, col, blk);
+    });
+    return true;
+  } else {
+    if (first_col && !wait_y()) return false;
+    fix_scatter<XCG>(a, idx, on, r, col, blk);
+    return true;
+  }
+}
+
 // One element of the collocated diffusion operator, FP64: fix_warps<Q>() warps, warp w on lines
 // 16 w .. 16 w + 15 of every direction.  A thread keeps its t-lines in registers (gather, pointwise
 // step, scatter: nodes t * Q^2 + line); r- and s-lines go through shared memory.  The FP64 pipe keeps
@@ -175,13 +192,11 @@ __device__ __forceinline__ void fix_block(const ApplyArgs &a, const OpTab<double
       for (int k = 0; k < 4; ++k)
         if (on[k]) ss[ls[k >> 1] + (k & 1) * 10] = w[k];
     }
-    const bool y_ok = col > col0 ? true : wait_y();
     __syncthreads();
-    if (!y_ok) return;
     double r[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) r[k] = on[k] ? y[k] + sr[at[k]] + ss[at[k]] : 0.0;
-    fix_scatter<XCG>(a, idx, on, r, col, blk);
+    if (!fix_turn<XCG>(a, idx, on, r, e, col, col == col0, blk, wait_y)) return;
     if (col + 1 < col1) __syncthreads();
   }
 }
@@ -312,9 +327,7 @@ __device__ __forceinline__ void fix_gauss_block(const ApplyArgs &a, const OpTab<
     __syncthreads();
     get(s0, v, P * P, Q, TP, t_part);
     fix_pass<Q, P>(M, v, w, full_bt);
-    const bool y_ok = col > col0 ? true : wait_y();
-    if (!y_ok) return;
-    fix_scatter<XCG>(a, idx, on, w, col, blk);
+    if (!fix_turn<XCG>(a, idx, on, w, e, col, col == col0, blk, wait_y)) return;
     if (col + 1 < col1) __syncthreads();
   }
 }
@@ -359,6 +372,12 @@ __global__ void __launch_bounds__(32 * fix_warps<Q>(), fix_min_blocks<P, Q>()) f
   ColourWait wait_y;
   colour_open_next();
   fix_any_block<P, Q, OP, false>(f.a, tab, f.tab, blockIdx.x, smem_raw, wait_y);
+}
+
+template <int P, int Q, int OP>
+__global__ void __launch_bounds__(APPLY_MAX_THREADS) fix_cluster_kernel(const FixArgs f, const OpTab<double> tab, const ClusterOrder order) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  fix_any_block<P, Q, OP, false>(f.a, tab, f.tab, blockIdx.x, smem_raw, order);
 }
 
 }  // namespace ceedgb
