@@ -129,7 +129,9 @@ __device__ __forceinline__ void colour_done(unsigned *done) {
 template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
 __device__ __noinline__ void batch_piece(const ApplyArgs &a, const uint32_t *fix, int64_t blk, const ColourOrder &wait_y) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
+  // one copy barrier per element slot of the largest block, idle slots included (apply_block readies them all):
+  // 64 at Q = 2, more than the APPLY_MAX_NE elements that a launch of its own may ask for
+  __shared__ uint64_t bar[STAGE ? (APPLY_MAX_THREADS + Q * Q - 1) / (Q * Q) : 1];
   const OpTab<T> &tab = *reinterpret_cast<const OpTab<T> *>(smem_raw);
   if constexpr (fix_covers<P, Q, OP, T>()) fix_any_block<P, Q, OP, false>(a, tab, fix, blk, smem_raw + batch_tab_bytes<T>(), wait_y);
   else apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blk, smem_raw + batch_tab_bytes<T>(), bar, wait_y);
@@ -254,6 +256,7 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
   b.grid_wait = grid_wait_limit();
   size_t smem = 0;
   const bool colloc = meshes[0]->Q == meshes[0]->P;
+  if (L.threads > APPLY_MAX_THREADS) return fail(CEED_ERR_INVALID, "batch blocks have at most 256 threads");
   for (int k = 0; k < n; ++k) {
     ceed_mesh_t m = meshes[k];
     if ((m->Q == m->P) != colloc) return fail(CEED_ERR_UNSUPPORTED, "a batch mixes quadrature rules");

@@ -93,3 +93,11 @@ def test_batch_rejects_bad_input(ceed):
         ceed.ceed_batch_create(meshes, qds, 0, cop, xs, xs)
     with pytest.raises(ceed.CeedError):      # BF16 batches are not supported
         ceed.ceed_batch_create(meshes, qds, 2, cop, xs, ys)
+
+
+@pytest.mark.parametrize("prec", [0, 1, 5])
+def test_batch_of_the_lowest_order(ceed, prec):
+    """p = 1 collocated: 64 elements (4 points a layer) per block, the most any order has.  Exactly one block's worth
+    of elements in a colour, one more, and one element alone; a higher order beside it in the same blocks."""
+    for dims in ((8, 8, 8), (13, 10, 4), (1, 1, 1)):
+        test_batch_matches_single_mesh_and_oracle(ceed, [(1, dims), (2, (3, 2, 2))], "gll", "diffusion", prec, 1, 2)
