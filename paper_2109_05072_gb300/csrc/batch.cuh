@@ -9,6 +9,7 @@
 #include <cstring>
 
 #include "apply_kernel.cuh"
+#include "progress.h"
 
 namespace ceedgb {
 
@@ -99,7 +100,7 @@ struct ColourOrder {
       int ok = 1;
       const volatile unsigned *v = prev;
       long long it = 0;
-      while (*v < target) {
+      while (!progress_reached(*v, target)) {
         if (++it > limit) {
           ok = 0;
           *err = CEED_ERR_TIMEOUT;

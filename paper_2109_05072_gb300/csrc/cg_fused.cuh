@@ -81,14 +81,15 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
     ApplyArgs a = g.a;
     a.dot_sh = &dsh;
     // pieces of work (element blocks) numbered colour by colour, every G-th one here (a fixed share:
-    // dsh adds them in a fixed order); the counters run on from one iteration to the next
+    // dsh adds them in a fixed order); the counters run on from one iteration to the next,
+    // modulo 2^32 (progress.h)
     int64_t base = 0;
     unsigned before = 0;  // pieces of the colour before
     for (int c = 0; c < g.ncolors; ++c) {
       a.e_begin = g.cstart[c];
       a.e_count = g.cstart[c + 1] - a.e_begin;
       const int64_t nwork = (a.e_count + a.ne - 1) / a.ne;
-      const ColourOrder wait_y{c ? g.done + (c - 1) * SYNC_LINE : nullptr, before * (unsigned)(it + 1), g.grid_wait, &sc->timeout, &ok_sh};
+      const ColourOrder wait_y{c ? g.done + (c - 1) * SYNC_LINE : nullptr, progress_target(before, (unsigned)it), g.grid_wait, &sc->timeout, &ok_sh};
       for (int64_t v = (blockIdx.x + G - base % G) % G; v < nwork; v += G) {
         if constexpr (fix_covers<P, Q, OP, T>()) fix_block<Q, true>(a, tab, g.fix, v, smem_raw, wait_y);
         else apply_block<P, Q, OP, T, TQ, false, true>(a, tab, v, smem_raw, nobar, wait_y);
