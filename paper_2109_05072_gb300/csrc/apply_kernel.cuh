@@ -621,8 +621,10 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
   const int el = tid / NPT;
   const int ij = tid - el * NPT;
   const int i = ij % Q, j = ij / Q;
-  const unsigned eb = (unsigned)blk / (unsigned)a.cgroups, cg = (unsigned)blk - eb * (unsigned)a.cgroups;
-  const int col0 = (int)cg * a.cpb, col1 = min(a.ncol, col0 + a.cpb);
+  // (XCG: the PCG iteration's one column)
+  const unsigned cgroups = XCG ? 1u : (unsigned)a.cgroups;
+  const unsigned eb = (unsigned)blk / cgroups, cg = (unsigned)blk - eb * cgroups;
+  const int col0 = XCG ? 0 : (int)cg * a.cpb, col1 = XCG ? 1 : min(a.ncol, col0 + a.cpb);
   const int64_t e = a.e_begin + (int64_t)eb * a.ne + el;
   const bool active = (el < a.ne) && (e < a.e_begin + a.e_count);
   const bool node_thread = (i < P) && (j < P);

@@ -82,14 +82,15 @@ __device__ __forceinline__ int64_t pieces(const BatchArgs<T> &b, int c, int m) {
   return (b.m[m].cstart[c + 1] - b.m[m].cstart[c] + a.ne - 1) / a.ne * a.cgroups;
 }
 
-// Order between the colours of a persistent apply without a grid barrier.  done[c] counts the pieces
-// of work (element blocks) of colour c that are in memory; a piece of colour c touches y once
-// done[c - 1] has reached its total -- every piece of colour c - 1 waited for colour c - 2, so all
+// Order between the colours of a persistent apply without a grid barrier.  done[c] counts the work of
+// colour c that is in memory: the batch's pieces (element blocks), or in the fused PCG iteration the blocks that
+// have finished their share of the colour.  Work of colour c touches y once
+// done[c - 1] has reached its total -- all of colour c - 1 waited for colour c - 2, so all
 // earlier colours are then in memory.  Blocks take pieces in colour order, so the earliest unfinished
 // piece never waits, and all that a piece does before its scatter (gather, contractions) overlaps the
 // colour before.  The wait is bounded like the grid barrier's.
 struct ColourOrder {
-  const unsigned *prev;   // counter of the colour before; null: nothing to wait for
+  const unsigned *prev;   // counter of the colour before; null: nothing to wait for, or waited for already
   unsigned target;
   long long limit;
   int *err;
@@ -116,7 +117,7 @@ struct ColourOrder {
   }
 };
 
-// The block's piece of work is done (its writes included): called by every thread.
+// The block's work counted here is done (its writes included): called by every thread.
 __device__ __forceinline__ void colour_done(unsigned *done) {
   __syncthreads();  // also frees shared memory for the next piece
   if (threadIdx.x == 0) {

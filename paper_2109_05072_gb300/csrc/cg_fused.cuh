@@ -81,23 +81,31 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
     ApplyArgs a = g.a;
     a.dot_sh = &dsh;
     // pieces of work (element blocks) numbered colour by colour, every G-th one here (a fixed share:
-    // dsh adds them in a fixed order); the counters run on from one iteration to the next,
-    // modulo 2^32 (progress.h)
+    // dsh adds them in a fixed order).  A block waits once per colour, at its first piece, and counts itself
+    // once, after its last; with a wait, a fence and a count at every piece its stores were waited for before the
+    // next one began.  p = 7, ms an iteration with grid barriers / counts at every piece / now: 64^3 FP32 3.47 /
+    // 4.13 / 3.34, double-float 6.02 / 6.11 / 6.00; 24^3 FP32 0.309 / 0.301 / 0.270; 16^3 FP32 0.154 / 0.123 /
+    // 0.119.  (A second code path for the later pieces that loads their old y with x was slower: 3.92 at 64^3.)
+    // The counters run on from one iteration to the next, modulo 2^32 (progress.h).
     int64_t base = 0;
-    unsigned before = 0;  // pieces of the colour before
+    unsigned before = 0;  // blocks that have pieces of the colour before
     for (int c = 0; c < g.ncolors; ++c) {
       a.e_begin = g.cstart[c];
       a.e_count = g.cstart[c + 1] - a.e_begin;
       const int64_t nwork = (a.e_count + a.ne - 1) / a.ne;
-      const ColourOrder wait_y{c ? g.done + (c - 1) * SYNC_LINE : nullptr, progress_target(before, (unsigned)it), g.grid_wait, &sc->timeout, &ok_sh};
-      for (int64_t v = (blockIdx.x + G - base % G) % G; v < nwork; v += G) {
+      const int64_t v0 = (blockIdx.x + G - base % G) % G;
+      const ColourOrder colour{c ? g.done + (c - 1) * SYNC_LINE : nullptr, progress_target(before, (unsigned)it), g.grid_wait,
+                               &sc->timeout, &ok_sh};
+      for (int64_t v = v0; v < nwork; v += G) {
+        if (v != v0) __syncthreads();  // shared memory is reused by the next piece
+        const ColourOrder wait_y = v == v0 ? colour : ColourOrder{};
         if constexpr (fix_covers<P, Q, OP, T>()) fix_block<Q, true>(a, tab, g.fix, v, smem_raw, wait_y);
         else apply_block<P, Q, OP, T, TQ, false, true>(a, tab, v, smem_raw, nobar, wait_y);
-        if (c && !ok_sh) return;
-        colour_done(g.done + c * SYNC_LINE);
+        if (c && v == v0 && !ok_sh) return;
       }
+      if (v0 < nwork) colour_done(g.done + c * SYNC_LINE);
       base += nwork;
-      before = (unsigned)nwork;
+      before = (unsigned)(nwork < G ? nwork : G);
     }
     if (tid == 0) g.part[blockIdx.x] = dsh;
     if (!grid_barrier(g.sync, &sc->timeout, g.grid_wait, &ok_sh)) return;
