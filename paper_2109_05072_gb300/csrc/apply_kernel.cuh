@@ -607,9 +607,12 @@ inline void column_split(ApplyArgs &a, int64_t eblocks) {
 // provides shared memory for ceil(blockDim / Q^2) elements and the mbarrier array.
 // XCG: x is read through L2 only (ld.global.cg) instead of the read-only path: required when x
 // changes during the kernel (the persistent CG iteration updates p between its applies).
+// SPLIT: false if a block does all columns of its elements (a.cgroups = 1).  A path of its own for the double-float
+// kernels, which run at their register cap: with the group's arithmetic in the way 64^3 at p = 7 took 3.42 ms, and
+// 24^3 at p = 8 0.585 (one column) and 2.46 ms (four), against 3.06, 0.517 and 2.13 without; the others gain nothing.
 // wait_y: called by every thread of the block before its first access to y (earlier colours written);
 // false if it gave up, and the block then writes nothing.
-template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool XCG = false, typename WaitY>
+template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool XCG = false, bool SPLIT = !XCG, typename WaitY>
 __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &tab, int64_t blk,
                                             unsigned char *smem_raw, uint64_t *bar, const WaitY &wait_y) {
   constexpr int NPT = Q * Q;
@@ -622,9 +625,9 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
   const int ij = tid - el * NPT;
   const int i = ij % Q, j = ij / Q;
   // (XCG: the PCG iteration's one column)
-  const unsigned cgroups = XCG ? 1u : (unsigned)a.cgroups;
+  const unsigned cgroups = SPLIT ? (unsigned)a.cgroups : 1u;
   const unsigned eb = (unsigned)blk / cgroups, cg = (unsigned)blk - eb * cgroups;
-  const int col0 = XCG ? 0 : (int)cg * a.cpb, col1 = XCG ? 1 : min(a.ncol, col0 + a.cpb);
+  const int col0 = SPLIT ? (int)cg * a.cpb : 0, col1 = XCG ? 1 : SPLIT ? min(a.ncol, col0 + a.cpb) : a.ncol;
   const int64_t e = a.e_begin + (int64_t)eb * a.ne + el;
   const bool active = (el < a.ne) && (e < a.e_begin + a.e_count);
   const bool node_thread = (i < P) && (j < P);
@@ -813,13 +816,13 @@ apply_kernel(const ApplyArgs a, const OpTab<T> tab) {
 // (dependent compensated sums, quadrature-data loads), so it is given more resident warps to switch
 // between instead of registers to hoist loads into (128: the best of 96..255 measured at p = 7).
 // Blocks of at most APPLY_MAX_THREADS threads.
-template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
+template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool SPLIT>
 __global__ void __maxnreg__(APPLY_DF_MAX_REGS) apply_kernel_capped(const ApplyArgs a, const OpTab<T> tab) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
   ColourWait wait_y;
   colour_open_next();
-  apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar, wait_y);
+  apply_block<P, Q, OP, T, TQ, STAGE, false, SPLIT>(a, tab, blockIdx.x, smem_raw, bar, wait_y);
 }
 
 // One colour's launch: the first of an application as any launch, the others as programmatic
@@ -897,10 +900,12 @@ template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
 int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne, cudaStream_t s) {
   const size_t smem = (size_t)ne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>();
   constexpr bool CAPPED = std::is_same<T, DF>::value;
-  const void *kfn;
-  if constexpr (CAPPED) kfn = (const void *)apply_kernel_capped<P, Q, OP, T, TQ, STAGE>;
-  else kfn = (const void *)apply_kernel<P, Q, OP, T, TQ, STAGE>;
-  if (int st = ensure_dynamic_smem(kfn, smem)) return st;
+  if constexpr (CAPPED) {
+    if (int st = ensure_dynamic_smem((const void *)apply_kernel_capped<P, Q, OP, T, TQ, STAGE, false>, smem)) return st;
+    if (int st = ensure_dynamic_smem((const void *)apply_kernel_capped<P, Q, OP, T, TQ, STAGE, true>, smem)) return st;
+  } else {
+    if (int st = ensure_dynamic_smem((const void *)apply_kernel<P, Q, OP, T, TQ, STAGE>, smem)) return st;
+  }
   const dim3 block(Q * Q * ne);
   ApplyArgs a;
   a.emap = m->d_emap;
@@ -931,7 +936,9 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
     column_split(a, (n + ne - 1) / ne);
     const dim3 grid((unsigned)((n + ne - 1) / ne * a.cgroups));
     int st;
-    if constexpr (CAPPED) st = launch_colour(apply_kernel_capped<P, Q, OP, T, TQ, STAGE>, grid, block, smem, s, first, a, tab);
+    if constexpr (CAPPED)
+      st = launch_colour(a.cgroups > 1 ? apply_kernel_capped<P, Q, OP, T, TQ, STAGE, true> : apply_kernel_capped<P, Q, OP, T, TQ, STAGE, false>,
+                         grid, block, smem, s, first, a, tab);
     else st = launch_colour(apply_kernel<P, Q, OP, T, TQ, STAGE>, grid, block, smem, s, first, a, tab);
     if (st) return st;
     first = false;
