@@ -127,9 +127,13 @@ __device__ __forceinline__ void colour_done(unsigned *done) {
 }
 
 // One piece of work of one order: a function of its own, so that the orders' register needs do not add up (inlined
-// together under the cap of 128 registers they spill 1.8 KB per thread; here 48 bytes at most).
+// together under the cap of 128 registers they spill 1.8 KB per thread; here 48 bytes at most).  It copies its arguments:
+// through the caller's references every use of one is a load from local memory (double-float, p = 3, 5, 7 on 48^3, 40^3,
+// 32^3 elements, 3 / 12 columns: 10.8 / 39.2 ms, 9.5 / 35.2 with copies).
 template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
-__device__ __noinline__ void batch_piece(const ApplyArgs &a, const uint32_t *fix, int64_t blk, const ColourOrder &wait_y) {
+__device__ __noinline__ void batch_piece(const ApplyArgs &args, const uint32_t *fix, int64_t blk, const ColourOrder &order) {
+  const ApplyArgs a = args;
+  const ColourOrder wait_y = order;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // one copy barrier per element slot of the largest block, idle slots included (apply_block readies them all):
   // 64 at Q = 2, more than the APPLY_MAX_NE elements that a launch of its own may ask for
@@ -302,8 +306,7 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     unsigned grid = (unsigned)(per_sm * nsm);
     if (L.grid > 0 && L.grid < grid) grid = L.grid;
     // cooperative launch: the runtime refuses it unless every block of the grid can be resident at
-    // once, which is what the grid barrier between colours relies on (the barrier's bounded wait
-    // stays as a second line of defence)
+    // once (pieces are taken in order, so the waits between colours end with fewer, too; they are bounded all the same)
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -319,7 +322,7 @@ int launch_batch(int n, ceed_mesh_t const *meshes, const ApplyReq *reqs, const O
     return CEED_OK;
   };
   // (the double-float operator included: unlike its single-mesh kernel it runs fastest without a
-  // register cap here -- 7.1 / 7.8 GDOF/s at 1 / 4 right-hand sides against 6.1 at 128 registers)
+  // register cap here -- 7.2 / 7.7 GDOF/s at 1 / 4 right-hand sides; 6.1 at 128 registers, the orders then inlined)
   if (colloc) return L.stage ? go(batch_kernel<OP, T, TQ, true, true>) : go(batch_kernel<OP, T, TQ, false, true>);
   return L.stage ? go(batch_kernel<OP, T, TQ, true, false>) : go(batch_kernel<OP, T, TQ, false, false>);
 }
