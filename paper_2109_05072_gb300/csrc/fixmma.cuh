@@ -15,8 +15,8 @@
 //    FP64 result: everything but the products runs on the integer pipe.
 // The error is that of a dot product with the line cut at 62 bits below its largest value and one
 // final rounding, smaller than that of the chain of FP64 FMAs (one rounding per term and fold).
-// A line that holds an infinity or a NaN, or whose largest value lies outside 2^-895 .. 2^877, takes plain
-// FP64 FMAs instead.
+// A line that holds an infinity or a NaN, or whose largest value is not zero and lies outside 2^-895 .. 2^877, takes
+// plain FP64 FMAs instead.
 //
 // Fragments: a warp holds 16 lines; lane 4 g + t owns entries 2t, 2t+1 of lines g and g + 8, on the way
 // in (A fragment: the digit of the pair as one half2) and on the way out (C fragment), so a pass
@@ -113,10 +113,12 @@ __device__ __forceinline__ double fix_out(const uint32_t (&u)[FIX_DIGITS], int e
 }
 
 // Biased exponent E of the largest of the values whose high words' magnitudes have the maximum m (64 for
-// all zero: every digit is then zero), and whether it lies outside the integer range.
+// all zero: every digit is then zero), and whether it lies outside the integer range (128 .. 1900).  High words all zero
+// are zeros or subnormals below 2^-1042; the latter (fix_tiny) lie outside as well.
 __device__ __forceinline__ int fix_exponent(int m) { return max(m >> 20, 64); }
-__device__ __forceinline__ bool fix_odd(int m) { return (m >> 20) > 1900 || (m != 0 && (m >> 20) < 128); }
+__device__ __forceinline__ bool fix_odd_or_zero(int m) { return (uint32_t)(m - (128 << 20)) >= (uint32_t)(1901 - 128) << 20; }
 __device__ __forceinline__ int fix_mag(double v) { return __double2hiint(v) & 0x7fffffff; }
+__device__ __forceinline__ bool fix_tiny(double v0, double v1) { return (__double2loint(v0) | __double2loint(v1)) != 0; }
 
 // maximum over the four lanes that hold a line
 __device__ __forceinline__ int fix_quad_max(int m) {
@@ -162,7 +164,10 @@ template <int NI, int NO, typename Full>
 __device__ __forceinline__ void fix_pass(const FixMat &M, const double (&v)[4], double (&out)[4], Full full) {
   const int m0 = fix_quad_max(max(fix_mag(v[0]), fix_mag(v[1]))), m1 = fix_quad_max(max(fix_mag(v[2]), fix_mag(v[3])));
   const int E0 = fix_exponent(m0), E1 = fix_exponent(m1);
-  if (__any_sync(0xffffffffu, fix_odd(m0) || fix_odd(m1))) {
+  // (in two steps: lines of zeros are common, and the second is left out where there is none)
+  if (__any_sync(0xffffffffu, fix_odd_or_zero(m0) || fix_odd_or_zero(m1)) &&
+      __any_sync(0xffffffffu, (fix_odd_or_zero(m0) && (m0 != 0 || fix_tiny(v[0], v[1]))) ||
+                                  (fix_odd_or_zero(m1) && (m1 != 0 || fix_tiny(v[2], v[3]))))) {
     const int lane = threadIdx.x & 31, t = lane & 3, q = lane & ~3;
     double r[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll 1

@@ -83,8 +83,15 @@ __global__ void __launch_bounds__(32 * NTF_WARPS, ntf_blocks(NC)) nt_fix_kernel(
     m1 = fix_quad_max(m1);
     E0 = fix_exponent(m0);
     E1 = fix_exponent(m1);
-    odd0 = fix_odd(m0);
-    odd1 = fix_odd(m1);
+    bool t0 = false, t1 = false;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      t0 |= fix_tiny(u[c][0], u[c][1]);
+      t1 |= fix_tiny(u[c][2], u[c][3]);
+    }
+    const int tiny0 = fix_quad_max(t0), tiny1 = fix_quad_max(t1);
+    odd0 = fix_odd_or_zero(m0) && (m0 != 0 || tiny0 != 0);
+    odd1 = fix_odd_or_zero(m1) && (m1 != 0 || tiny1 != 0);
     odd = __any_sync(0xffffffffu, odd0 || odd1);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -175,7 +182,19 @@ __global__ void __launch_bounds__(32 * NTF_WARPS, ntf_blocks(NC)) nt_fix_kernel(
     }
     m0 = fix_quad_max(m0);
     m1 = fix_quad_max(m1);
-    const bool o0 = fix_odd(m0), o1 = fix_odd(m1);
+    bool o0 = fix_odd_or_zero(m0), o1 = fix_odd_or_zero(m1);
+    const bool any_o = __any_sync(0xffffffffu, o0 || o1);
+    if (any_o) {  // every lane of the warp
+      bool t0 = false, t1 = false;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        t0 |= fix_tiny(v[d][0], v[d][1]);
+        t1 |= fix_tiny(v[d][2], v[d][3]);
+      }
+      const int tiny0 = fix_quad_max(t0), tiny1 = fix_quad_max(t1);
+      o0 = o0 && (m0 != 0 || tiny0 != 0);
+      o1 = o1 && (m1 != 0 || tiny1 != 0);
+    }
     {
       const int F0 = fix_exponent(m0), F1 = fix_exponent(m1);
       uint32_t x0[D][8], x1[D][8];
@@ -204,7 +223,7 @@ __global__ void __launch_bounds__(32 * NTF_WARPS, ntf_blocks(NC)) nt_fix_kernel(
         }
       }
     }
-    if (__any_sync(0xffffffffu, o0 || o1)) {
+    if (any_o) {
 #pragma unroll
       for (int d = 0; d < D; ++d)
 #pragma unroll 1
