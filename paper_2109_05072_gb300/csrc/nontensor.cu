@@ -247,17 +247,15 @@ __device__ __forceinline__ void nt_pointwise(const T *__restrict__ qd, int64_t c
 // quadrature data read coalesced (element fastest), and the transposed contraction accumulated
 // in registers (node rows spread over the warps).  Output: the element vectors, [P][E].
 template <typename T, int D>
-__global__ void __launch_bounds__(NT_NE * NT_WARPS)
-    nt_fused_kernel(int64_t E, int64_t Es, int P, int Q, const uint32_t *__restrict__ rmap, const double *__restrict__ x,
-                    const T *__restrict__ tab, const T *__restrict__ qd, T *__restrict__ Ye, int masked) {
+__device__ __forceinline__ void nt_fused_block(int64_t e, bool valid, int64_t E, int64_t Es, int P, int Q,
+                                               const uint32_t *__restrict__ rmap, const double *__restrict__ x,
+                                               const T *__restrict__ tab, const T *__restrict__ qd, T *__restrict__ Ye, int masked) {
   extern __shared__ __align__(16) unsigned char nt_smem[];
   T *Us = reinterpret_cast<T *>(nt_smem);   // [P][NT_NE]
   T *Gc = Us + P * NT_NE;                    // [D][NT_QC][P]
   T *Sv = Gc + D * NT_QC * P;                // [D NT_QC][NT_NE + 1]
   constexpr int LD = NT_NE + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t e = (int64_t)blockIdx.x * NT_NE + lane;
-  const bool valid = e < E;
   for (int n = warp; n < P; n += NT_WARPS) {
     T v = T(0);
     if (valid) {
@@ -325,6 +323,28 @@ __global__ void __launch_bounds__(NT_NE * NT_WARPS)
       const int n = warp + NT_WARPS * j;
       if (n < P) Ye[(int64_t)n * E + e] = yr[j];
     }
+  }
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(NT_NE * NT_WARPS)
+    nt_fused_kernel(int64_t E, int64_t Es, int P, int Q, const uint32_t *__restrict__ rmap, const double *__restrict__ x,
+                    const T *__restrict__ tab, const T *__restrict__ qd, T *__restrict__ Ye, int masked) {
+  const int64_t e = (int64_t)blockIdx.x * NT_NE + (threadIdx.x & 31);
+  nt_fused_block<T, D>(e, e < E, E, Es, P, Q, rmap, x, tab, qd, Ye, masked);
+}
+
+// The same for the listed elements: list[0] of them from list[1] on (nontensor_fix.cu).
+template <int D>
+__global__ void __launch_bounds__(NT_NE * NT_WARPS)
+    nt_fused_list_kernel(const uint32_t *__restrict__ list, int64_t E, int64_t Es, int P, int Q, const uint32_t *__restrict__ rmap,
+                         const double *__restrict__ x, const double *__restrict__ tab, const double *__restrict__ qd,
+                         double *__restrict__ Ye, int masked) {
+  const int64_t n = list[0];
+  for (int64_t i0 = (int64_t)blockIdx.x * NT_NE; i0 < n; i0 += (int64_t)gridDim.x * NT_NE) {
+    const int64_t i = i0 + (threadIdx.x & 31);
+    nt_fused_block<double, D>(i < n ? list[1 + i] : 0, i < n, E, Es, P, Q, rmap, x, tab, qd, Ye, masked);
+    __syncthreads();  // shared memory is reused
   }
 }
 
@@ -491,6 +511,17 @@ static int launch_fused(ceed_nt_t h, const T *tab, const T *qd, const double *x,
   return CEED_OK;
 }
 
+// The elements that the slice kernel left (none, as a rule): at most two blocks for every SM.
+template <int D>
+static int launch_fused_list(ceed_nt_t h, const double *tab, const double *qd, const double *x, double *Ye, int masked, cudaStream_t s) {
+  const size_t sm = nt_fused_smem(h->P, D, sizeof(double));
+  if (int st = ensure_dynamic_smem((const void *)nt_fused_list_kernel<D>, 227 * 1024)) return st;
+  const unsigned grid = (unsigned)std::min<int64_t>((h->E + NT_NE - 1) / NT_NE, 304);
+  nt_fused_list_kernel<D><<<grid, NT_NE * NT_WARPS, sm, s>>>(h->d_again, h->E, h->Es, h->P, h->Q, h->d_rmap, x, tab, qd, Ye, masked);
+  CEED_CUDA_CHECK(cudaGetLastError());
+  return CEED_OK;
+}
+
 static int blas_fail(cublasStatus_t st, const char *where) {
   return fail(st == CUBLAS_STATUS_ALLOC_FAILED ? CEED_ERR_OOM : CEED_ERR_CUDA,
               std::string(where) + ": cuBLAS status " + std::to_string((int)st));
@@ -551,11 +582,16 @@ static int nt_apply_t(ceed_nt_t h, const NtChoice &c, const T *tab, const T *qd,
   T *Ye = reinterpret_cast<T *>(h->d_evec);
   int st;
   if (c.algo == CEED_NT_FUSED) {
-    if (std::is_same<T, double>::value && nt_fix_supported(h->P))
-      st = nt_fix_apply(h, D == 1 ? CEED_OP_MASS : CEED_OP_DIFFUSION, reinterpret_cast<const double *>(qd), x,
+    const int op = D == 1 ? CEED_OP_MASS : CEED_OP_DIFFUSION;
+    if (std::is_same<T, double>::value && nt_fix_supported(h, op)) {
+      st = nt_fix_apply(h, op, reinterpret_cast<const double *>(qd), x,
                         reinterpret_cast<double *>(Ye), masked, s);
-    else
+      if (st == CEED_OK)
+        st = launch_fused_list<D>(h, reinterpret_cast<const double *>(tab), reinterpret_cast<const double *>(qd), x,
+                                  reinterpret_cast<double *>(Ye), masked, s);
+    } else {
       st = launch_fused<T, D>(h, tab, qd, x, Ye, masked, s);
+    }
   } else if (c.algo == CEED_NT_TC) {
     if (sizeof(T) != 4) return fail(CEED_ERR_UNSUPPORTED, "tensor-core algorithm: F32 only");
     st = nt_tc_apply(h, D == 1 ? CEED_OP_MASS : CEED_OP_DIFFUSION, reinterpret_cast<const float *>(qd), x,
@@ -652,6 +688,7 @@ struct NtFree {
     cudaFree(h->d_tc_tab[1]);
     cudaFree(h->d_fix[0]);
     cudaFree(h->d_fix[1]);
+    cudaFree(h->d_again);
     delete h;
   }
 };
@@ -765,8 +802,7 @@ extern "C" int ceed_nt_setup(const ceed_nt_desc *desc, ceed_nt_t *out, void *str
   CEED_CUDA_CHECK(cudaMemcpyAsync(h->d_dir, dir.data(), (size_t)nL, cudaMemcpyHostToDevice, s));
   CEED_CUDA_CHECK(cudaMemcpyAsync(h->d_vert, desc->vertices, (size_t)E * 96, cudaMemcpyDeviceToDevice, s));
   CEED_CUDA_CHECK(cudaMemsetAsync(h->d_err, 0, sizeof(int), s));
-  if (nt_fix_supported(P))
-    if (int st = nt_fix_prepare(h.get(), tab64.data(), s)) return st;
+  if (int st = nt_fix_prepare(h.get(), tab64.data(), s)) return st;
   cublasStatus_t bs = cublasCreate(&h->blas);
   if (bs != CUBLAS_STATUS_SUCCESS) {
     h->blas = nullptr;

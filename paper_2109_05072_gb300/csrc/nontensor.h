@@ -46,8 +46,9 @@ struct ceed_nt_s {
   void *d_s = nullptr;
   float *d_tc_tab[2] = {nullptr, nullptr};  // tensor-core tables per op (mass, diffusion), see nontensor_tc.cu
   int tc_nchunk = 0;
-  uint32_t *d_fix[2] = {nullptr, nullptr};  // digit tables of the FP64 slice kernel per op, see nontensor_fix.cu
-  int fix_scale[2] = {0, 0};
+  uint32_t *d_fix[2] = {nullptr, nullptr};  // digit tables of the FP64 slice kernel per op where it serves, see nontensor_fix.cu
+  uint32_t *d_again = nullptr;              // [1 + E] number and list of the elements it leaves to the CUDA-core kernel
+  int fix_scale[2][2] = {};                 // their scales: forward, transposed
   cublasHandle_t blas = nullptr;
   ceedgb::NtChoice choice[2][3];  // [op][prec: 0 F64, 1 F32, 2 F64_DF (fused only)]
 };
@@ -59,7 +60,7 @@ int nt_tc_prepare(ceed_nt_t h);   // builds the chunked split tables of both ope
 int nt_tc_apply(ceed_nt_t h, int op, const float *qd, const double *x, float *Ye, int masked, cudaStream_t s);
 // FP64 fused operator on the tensor cores by exact integer slices (nontensor_fix.cu).
 constexpr int NTF_MAX_P = 35;   // integer sums over more nodes could leave FP32's exact range
-bool nt_fix_supported(int P);
+bool nt_fix_supported(ceed_nt_t h, int op);
 int nt_fix_prepare(ceed_nt_t h, const double *tab64, cudaStream_t s);
 int nt_fix_apply(ceed_nt_t h, int op, const double *qd, const double *x, double *Ye, int masked, cudaStream_t s);
 }  // namespace ceedgb
