@@ -163,6 +163,11 @@ int ceed_apply_host(ceed_mesh_t mesh, int op, const void *qdata, int prec, const
  * or direct loads), and the brick kernel with and without staging where the mesh and precision
  * allow it (ceed_set_apply_variant) -- on the caller's qdata, x and y (y is overwritten), times each with CUDA
  * events on `stream`, and keeps the fastest in the handle for (op, prec); later applies use it.
+ * On a small mesh the default is timed as well: elements times columns that fit one thread-block
+ * cluster of 8 blocks run all colours in one launch (reported as its elements per block, stage 1).
+ * FP64 operators on the integer slices -- collocated diffusion with 6 to 8 points per direction,
+ * mass and diffusion with 7 or 8 Gauss points -- have one kernel and no variants: the call times it,
+ * reports ne = 1, stage = 0 and keeps the default.
  * Returns the choice and its time per application.  Synchronizes `stream`. */
 int ceed_autotune_apply(ceed_mesh_t mesh, int op, const void *qdata, int prec, const double *x, double *y,
                         int nrhs, int32_t *best_ne, int32_t *best_stage, float *best_ms, void *stream);
@@ -175,7 +180,9 @@ int ceed_autotune_apply(ceed_mesh_t mesh, int op, const void *qdata, int prec, c
  * element variants (stages 0, 1) give bitwise-identical results; the brick variants add the
  * contributions to a shared node in another order (the brick's elements first), so they agree
  * with them to FP32 rounding, deterministically.  A brick choice applies to single-column applies;
- * several columns run the default element variant. */
+ * several columns run the default element variant.  A variant set here launches one kernel per
+ * colour; only the default may run a small mesh as one cluster (same bits).  FP64 operators on the
+ * integer slices (see ceed_autotune_apply) accept a variant and run their one kernel. */
 int ceed_set_apply_variant(ceed_mesh_t mesh, int op, int prec, int ne, int stage);
 
 /* Jacobi diagonal of the operator (the cheap preconditioner for CG, Section 1), FP64
@@ -524,7 +531,7 @@ int ceed_dot_noalloc(const double *x, const double *y, int64_t n, double *out, v
 int ceed_mesh_status(ceed_mesh_t mesh, void *stream);
 
 /* Limits of the bounded device-side waits (not an operation of the paper; failure handling):
- * copy_polls governs each apply kernel's wait for its quadrature-data copy (negative: the default
+ * copy_polls governs each staging apply kernel's wait for its quadrature-data copy (negative: the default
  * bound of 2^22 polls; 0: give up at once; the kernels keep that bound a compile-time constant, so
  * other values are INVALID), barrier_polls the grid barriers of the persistent batched launch and of
  * the fused CG iteration (negative: the default 2^25 polls; 0 .. 2^25: that many polls).  A wait

@@ -149,8 +149,6 @@ struct ColourWait {
 // A mesh small enough for one thread-block cluster: all its colours in one launch.  Every block gathers and
 // computes its elements at once, then the colours take turns at y, a cluster barrier between them (y is
 // read and written through L2).
-constexpr int CLUSTER_BLOCKS = 8;
-constexpr int CLUSTER_COLORS = 16;
 struct ClusterOrder {
   int ncolors;
   int start[CLUSTER_COLORS + 1];   // colour-sorted element ranges
@@ -857,15 +855,6 @@ __global__ void __launch_bounds__(APPLY_MAX_THREADS) apply_cluster_kernel(const 
   apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar, order);
 }
 
-// Elements per block if the mesh's elements times the columns fit one cluster (at most max_ne elements a block), else 0.
-// The rule is the launch's own limit: up to there one launch beats eight overlapping ones (64 elements at p = 2: 13 to 16 us against
-// 24.8).
-inline int cluster_elems(ceed_mesh_t m, const ApplyReq &r, int max_ne) {
-  if (r.dot_part || r.ncol > CLUSTER_BLOCKS || m->n_colors > CLUSTER_COLORS) return 0;
-  const int64_t per_column = CLUSTER_BLOCKS / r.ncol, ne = (m->E + per_column - 1) / per_column;
-  return ne <= max_ne ? (int)ne : 0;
-}
-
 // Launch `kernel` as one cluster over all colours (a.ne elements and one column per block).
 template <typename Kernel, typename Args, typename Tab>
 int launch_cluster(ceed_mesh_t m, Kernel kernel, ApplyArgs &a, const Args &args, const Tab &tab, int threads, size_t smem, cudaStream_t s) {
@@ -895,9 +884,10 @@ int launch_cluster(ceed_mesh_t m, Kernel kernel, ApplyArgs &a, const Args &args,
   return CEED_OK;
 }
 
-// Launch one kernel per colour for a fixed (P, Q, op, T, TQ) and variant (elements per block, staging).
+// Launch one kernel per colour for a fixed (P, Q, op, T, TQ) and variant (elements per block, staging); with the default
+// variant (by_default) one cluster over all colours where the mesh fits it.
 template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
-int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne, cudaStream_t s) {
+int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne, bool by_default, cudaStream_t s) {
   const size_t smem = (size_t)ne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>();
   constexpr bool CAPPED = std::is_same<T, DF>::value;
   if constexpr (CAPPED) {
@@ -921,11 +911,14 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
   a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
   a.dot_base = 0;
   a.dot_sh = nullptr;
-  if (const int cne = cluster_elems(m, r, std::min(max_elems_per_block<Q>(), APPLY_MAX_NE))) {
-    a.ne = cne;
-    if (r.dot_n) *r.dot_n = 0;
-    return launch_cluster(m, apply_cluster_kernel<P, Q, OP, T, TQ, STAGE>, a, a, tab, Q * Q * cne,
-                          (size_t)cne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>(), s);
+  if constexpr (STAGE) {
+    const int cne = by_default && !r.dot_part ? cluster_elems(m->E, m->n_colors, r.ncol, std::min(max_elems_per_block<Q>(), APPLY_MAX_NE)) : 0;
+    if (cne > 0) {
+      a.ne = cne;
+      if (r.dot_n) *r.dot_n = 0;
+      return launch_cluster(m, apply_cluster_kernel<P, Q, OP, T, TQ, STAGE>, a, a, tab, Q * Q * cne,
+                            (size_t)cne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>(), s);
+    }
   }
   bool first = true;
   for (int c = 0; c < m->n_colors; ++c) {
@@ -970,7 +963,8 @@ int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaS
   a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
   a.dot_base = 0;
   a.dot_sh = nullptr;
-  if (const int cne = cluster_elems(m, r, APPLY_MAX_THREADS / (32 * fix_warps<Q>()))) {
+  const int cne = r.dot_part ? 0 : cluster_elems(m->E, m->n_colors, r.ncol, APPLY_MAX_THREADS / (32 * fix_warps<Q>()));
+  if (cne > 0) {
     a.ne = cne;
     if (r.dot_n) *r.dot_n = 0;
     return launch_cluster(m, fix_cluster_kernel<P, Q, OP>, a, f, tab, 32 * fix_warps<Q>() * cne, cne * fix_smem<P, Q, OP>(), s);
@@ -994,10 +988,12 @@ int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaS
 template <int P, int Q, int OP, typename T, typename TQ>
 int launch_colours(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, cudaStream_t s) {
   int ne = r.ne, stage = r.stage;
-  if (ne <= 0) {  // autotuned choice for this (op, precision), else the default
+  bool by_default = false;
+  if (ne <= 0) {  // the variant set or tuned for this (op, precision), else the default
     const ApplyChoice &ch = m->tuned[r.op][r.prec];
-    ne = ch.ne > 0 ? ch.ne : default_elems_per_block<Q>();
-    stage = ch.ne > 0 ? ch.stage : 1;
+    by_default = ne < 0 || ch.ne <= 0;
+    ne = by_default ? default_elems_per_block<Q>() : ch.ne;
+    stage = by_default ? 1 : ch.stage;
   }
   if (stage >= 2) {  // brick kernel: FP32-pipe operators on a brick lattice, one column
     if constexpr (std::is_same<T, float>::value) {
@@ -1009,14 +1005,12 @@ int launch_colours(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, cudaSt
     if (r.ne > 0) return fail(CEED_ERR_UNSUPPORTED, "brick kernel: needs a brick lattice, one column, an FP32-pipe operator");
     ne = default_elems_per_block<Q>();  // a tuned brick choice on a request the bricks cannot serve
     stage = 1;
+    by_default = true;
   }
   if (ne > max_elems_per_block<Q>() || ne > APPLY_MAX_NE) return fail(CEED_ERR_INVALID, "elements per block too large");
-  if constexpr (fix_covers<P, Q, OP, T>()) {
-    return launch_fix<P, Q, OP>(m, tab, r, s);
-  } else {
-  if (stage) return launch_variant<P, Q, OP, T, TQ, true>(m, tab, r, ne, s);
-  return launch_variant<P, Q, OP, T, TQ, false>(m, tab, r, ne, s);
-  }
+  if constexpr (fix_covers<P, Q, OP, T>()) return launch_fix<P, Q, OP>(m, tab, r, s);
+  else if (stage) return launch_variant<P, Q, OP, T, TQ, true>(m, tab, r, ne, by_default, s);
+  else return launch_variant<P, Q, OP, T, TQ, false>(m, tab, r, ne, by_default, s);
 }
 
 // Dispatch on (P, collocated?) for one (op, T, TQ).

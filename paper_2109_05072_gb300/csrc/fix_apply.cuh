@@ -340,9 +340,7 @@ __device__ __forceinline__ void fix_gauss_block(const ApplyArgs &a, const OpTab<
 // integer pipe; 5: 10 against 8 and the tile's unused lines); longer ones do not fit the tile.
 template <int P, int Q, int OP, typename T>
 constexpr bool fix_covers() {
-  return std::is_same<T, double>::value &&
-         ((OP == CEED_OP_DIFFUSION && P == Q && Q >= FIX_MIN_Q && Q <= FIX_MAX_Q) ||
-          ((OP == CEED_OP_DIFFUSION || OP == CEED_OP_MASS) && Q == P + 1 && Q > FIX_MIN_Q && Q <= FIX_MAX_Q));
+  return std::is_same<T, double>::value && slice_operator(P, Q, OP);
 }
 
 template <int P, int Q, int OP, bool XCG, typename WaitY>

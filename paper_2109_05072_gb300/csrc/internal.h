@@ -99,6 +99,20 @@ struct CgScalars {
 constexpr int FIX_DIGITS = 8;
 constexpr int FIX_TAB_WORDS = FIX_DIGITS * 32 + 32;
 constexpr int FIX_MIN_Q = 6, FIX_MAX_Q = 8;  // points per direction the slice kernel covers
+// FP64 operators that run on the slices (the reasons at fix_apply.cuh), whatever variant of the apply is asked for.
+constexpr bool slice_operator(int P, int Q, int op) {
+  return (op == CEED_OP_DIFFUSION && P == Q && Q >= FIX_MIN_Q && Q <= FIX_MAX_Q) ||
+         ((op == CEED_OP_DIFFUSION || op == CEED_OP_MASS) && Q == P + 1 && Q > FIX_MIN_Q && Q <= FIX_MAX_Q);
+}
+
+// One-cluster launch of small meshes (apply_kernel.cuh): elements per block if the elements times the columns fit (at most
+// max_ne elements a block), else 0.
+constexpr int CLUSTER_BLOCKS = 8, CLUSTER_COLORS = 16;
+inline int cluster_elems(int64_t E, int n_colors, int ncol, int max_ne) {
+  if (ncol > CLUSTER_BLOCKS || n_colors > CLUSTER_COLORS) return 0;
+  const int64_t per_column = CLUSTER_BLOCKS / ncol, ne = (E + per_column - 1) / per_column;
+  return ne <= max_ne ? (int)ne : 0;
+}
 
 // A value's eight balanced base-256 digits as FP16 bit patterns, leading digit first: the integer nearest
 // to v 2^scale, which has to lie below 2^62 (mesh.cu).
@@ -197,7 +211,7 @@ struct ApplyReq {
   double *y;
   int ncol;          // ncomp * nrhs
   int masked;
-  int ne = 0;        // > 0: force this many elements per block (autotuner), else tuned/default
+  int ne = 0;        // > 0: this many elements per block (autotuner); 0: the tuned or set variant, else the default; < 0: the default
   int stage = 1;     // with ne > 0: staging switch
   double *dot_part = nullptr;  // non-null (ncol = 1): per-block partial sums of x . y over final node values
   int64_t *dot_n = nullptr;    // out: number of partial sums written

@@ -764,7 +764,9 @@ static bool brick_ok(ceed_mesh_t m, int prec, int ncol) {
 
 // ---------------------------------------------------------------------------------------------
 // Autotuner for the apply kernel: times every (elements per block, staging) variant on the
-// caller's mesh, quadrature data and vectors, and keeps the fastest for (op, prec) in the handle.
+// caller's mesh, quadrature data and vectors, and keeps the fastest for (op, prec) in the handle.  The default is timed
+// too where it is a launch of its own: one cluster for a small mesh.  An operator on the integer slices has
+// no variants: there is nothing to choose, and the default stays.
 extern "C" int ceed_autotune_apply(ceed_mesh_t m, int op, const void *qdata, int prec, const double *x, double *y,
                                    int nrhs, int32_t *best_ne, int32_t *best_stage, float *best_ms, void *stream) {
   if (int st = check_mesh(m)) return st;
@@ -786,34 +788,48 @@ extern "C" int ceed_autotune_apply(ceed_mesh_t m, int op, const void *qdata, int
   CEED_CUDA_CHECK(cudaEventCreate(&e1));
   ApplyChoice best;
   best.ms = 1e30f;
+  int32_t report_ne = 0, report_stage = 0;
   const int reps = 3;
+  const auto time = [&](int ne, int stage) {  // ms of one application, or -1
+    r.ne = ne;
+    r.stage = stage;
+    if (launch_apply(m, r, s) != CEED_OK) return -1.f;  // e.g. shared memory beyond the limit
+    cudaEventRecord(e0, s);
+    for (int k = 0; k < reps; ++k) launch_apply(m, r, s);
+    cudaEventRecord(e1, s);
+    if (cudaEventSynchronize(e1) != cudaSuccess) return -1.f;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    return ms / reps;
+  };
+  const bool slices = prec == CEED_F64 && slice_operator(m->P, m->Q, op);
+  const int cluster = cluster_elems(m->E, m->n_colors, r.ncol, ne_max);
+  if (slices || cluster > 0) {
+    const float ms = time(-1, 1);
+    if (ms > 0.f) {
+      best.ms = ms;  // best.ne = 0: the default
+      report_ne = slices ? 1 : cluster;
+      report_stage = slices ? 0 : 1;
+    }
+  }
   const bool bricks = brick_ok(m, prec, r.ncol);
-  for (int stage = 0; stage <= (bricks ? 3 : 1); ++stage) {
+  for (int stage = 0; !slices && stage <= (bricks ? 3 : 1); ++stage) {
     for (int ne = 1; ne <= (stage >= 2 ? 1 : ne_max); ne *= 2) {  // the brick kernel has one shape
-      r.ne = ne;
-      r.stage = stage;
-      if (launch_apply(m, r, s) != CEED_OK) continue;  // e.g. shared memory beyond the limit
-      cudaEventRecord(e0, s);
-      for (int k = 0; k < reps; ++k) launch_apply(m, r, s);
-      cudaEventRecord(e1, s);
-      if (cudaEventSynchronize(e1) != cudaSuccess) break;
-      float ms = 0.f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      ms /= reps;
-      if (ms < best.ms) {
+      const float ms = time(ne, stage);
+      if (ms > 0.f && ms < best.ms) {
         best.ms = ms;
-        best.ne = ne;
-        best.stage = stage;
+        best.ne = report_ne = ne;
+        best.stage = report_stage = stage;
       }
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   CEED_CUDA_CHECK(cudaGetLastError());
-  if (best.ne == 0) return fail(CEED_ERR_CUDA, "no apply variant ran");
+  if (report_ne == 0) return fail(CEED_ERR_CUDA, "no apply variant ran");
   m->tuned[op][prec] = best;
-  if (best_ne) *best_ne = best.ne;
-  if (best_stage) *best_stage = best.stage;
+  if (best_ne) *best_ne = report_ne;
+  if (best_stage) *best_stage = report_stage;
   if (best_ms) *best_ms = best.ms;
   return CEED_OK;
 }
