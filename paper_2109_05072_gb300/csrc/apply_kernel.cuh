@@ -855,7 +855,9 @@ __global__ void __launch_bounds__(APPLY_MAX_THREADS) apply_cluster_kernel(const 
   apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar, order);
 }
 
-// Launch `kernel` as one cluster over all colours (a.ne elements and one column per block).
+// Launch `kernel` as one cluster over all colours (a.ne elements and one column per block).  CLUSTER_REFUSED: the device
+// cannot place such a cluster (a partition of it may hold fewer SMs); the caller launches per colour.
+constexpr int CLUSTER_REFUSED = -1;
 template <typename Kernel, typename Args, typename Tab>
 int launch_cluster(ceed_mesh_t m, Kernel kernel, ApplyArgs &a, const Args &args, const Tab &tab, int threads, size_t smem, cudaStream_t s) {
   ClusterOrder order;
@@ -880,8 +882,10 @@ int launch_cluster(ceed_mesh_t m, Kernel kernel, ApplyArgs &a, const Args &args,
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  CEED_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, args, tab, order));
-  return CEED_OK;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args, tab, order);
+  if (e == cudaSuccess) return CEED_OK;
+  cudaGetLastError();  // the launches per colour report what else may be wrong
+  return CLUSTER_REFUSED;
 }
 
 // Launch one kernel per colour for a fixed (P, Q, op, T, TQ) and variant (elements per block, staging); with the default
@@ -916,8 +920,10 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
     if (cne > 0) {
       a.ne = cne;
       if (r.dot_n) *r.dot_n = 0;
-      return launch_cluster(m, apply_cluster_kernel<P, Q, OP, T, TQ, STAGE>, a, a, tab, Q * Q * cne,
-                            (size_t)cne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>(), s);
+      const int st = launch_cluster(m, apply_cluster_kernel<P, Q, OP, T, TQ, STAGE>, a, a, tab, Q * Q * cne,
+                                    (size_t)cne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>(), s);
+      if (st != CLUSTER_REFUSED) return st;
+      a.ne = ne;
     }
   }
   bool first = true;
@@ -967,7 +973,9 @@ int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaS
   if (cne > 0) {
     a.ne = cne;
     if (r.dot_n) *r.dot_n = 0;
-    return launch_cluster(m, fix_cluster_kernel<P, Q, OP>, a, f, tab, 32 * fix_warps<Q>() * cne, cne * fix_smem<P, Q, OP>(), s);
+    const int st = launch_cluster(m, fix_cluster_kernel<P, Q, OP>, a, f, tab, 32 * fix_warps<Q>() * cne, cne * fix_smem<P, Q, OP>(), s);
+    if (st != CLUSTER_REFUSED) return st;
+    a.ne = 1;
   }
   bool first = true;
   for (int c = 0; c < m->n_colors; ++c) {
