@@ -948,7 +948,7 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
   return CEED_OK;
 }
 
-// The slice kernel: one element per block, one launch per colour.
+// The slice kernel: one element per block, one launch per colour (nothing staged, so no copy to wait for).
 template <int P, int Q, int OP>
 int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaStream_t s) {
   constexpr size_t smem = fix_smem<P, Q, OP>();
@@ -963,8 +963,6 @@ int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaS
   a.ncol = r.ncol;
   a.masked = r.masked;
   a.ne = 1;
-  a.err = m->d_err + 1;
-  a.wait_limit = copy_wait_limit();
   a.estride = qdata_estride(OP, sizeof(double), Q);
   a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
   a.dot_base = 0;
