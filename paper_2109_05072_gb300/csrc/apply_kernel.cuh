@@ -589,9 +589,11 @@ struct ApplyArgs {
 // a colour with few element blocks leaves the chip idle while each of them walks all the columns, and
 // a block that still has columns to do holds up the colours behind it.  So columns are spread
 // over blocks until a colour has COLUMN_BLOCKS of them (about 16 per SM, more than are resident); the
-// repeated quadrature data comes from L2.  p = 3 Gauss, 848
-// elements a colour, 12 columns: 1.65 ms with all columns in a block, 2.00 so with overlapping colours (their waiting
-// blocks take the working ones' places), 1.28 ms spread.
+// repeated quadrature data comes from L2.  p = 3 Gauss, 848 elements a colour, 12 columns: 1.65 ms with all columns in a
+// block, 2.00 so with overlapping colours (their waiting blocks take the working ones' places), 1.17 spread.  Eleven
+// shapes from 27 to 3,375 elements a colour, 3 to 12 columns, p = 2 to 7, all precisions, with 1, 4, 16 and 64
+// blocks per SM in this place: 16 is within 5% of the best in ten (30^3, p = 3, 4 columns: 758, 757, 467, 467 us) and
+// 12% behind 64 in one (24^3, p = 5, 4 columns: 954 against 854).
 constexpr int64_t COLUMN_BLOCKS = 152 * 16;
 inline void column_split(ApplyArgs &a, int64_t eblocks) {
   const int64_t groups = std::min<int64_t>(a.ncol, std::max<int64_t>(1, COLUMN_BLOCKS / std::max<int64_t>(1, eblocks)));
@@ -916,7 +918,7 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
   a.dot_base = 0;
   a.dot_sh = nullptr;
   if constexpr (STAGE) {
-    const int cne = by_default && !r.dot_part ? cluster_elems(m->E, m->n_colors, r.ncol, std::min(max_elems_per_block<Q>(), APPLY_MAX_NE)) : 0;
+    const int cne = by_default && !r.dot_part ? cluster_elems(m->E, m->n_colors, r.ncol, cluster_max_elems(std::is_same<T, double>::value, false, Q)) : 0;
     if (cne > 0) {
       a.ne = cne;
       if (r.dot_n) *r.dot_n = 0;
@@ -967,7 +969,7 @@ int launch_fix(ceed_mesh_t m, const OpTab<double> &tab, const ApplyReq &r, cudaS
   a.dot_part = (r.ncol == 1) ? r.dot_part : nullptr;
   a.dot_base = 0;
   a.dot_sh = nullptr;
-  const int cne = r.dot_part ? 0 : cluster_elems(m->E, m->n_colors, r.ncol, APPLY_MAX_THREADS / (32 * fix_warps<Q>()));
+  const int cne = r.dot_part ? 0 : cluster_elems(m->E, m->n_colors, r.ncol, cluster_max_elems(true, true, Q));
   if (cne > 0) {
     a.ne = cne;
     if (r.dot_n) *r.dot_n = 0;

@@ -106,8 +106,18 @@ constexpr bool slice_operator(int P, int Q, int op) {
 }
 
 // One-cluster launch of small meshes (apply_kernel.cuh): elements per block if the elements times the columns fit (at most
-// max_ne elements a block), else 0.
+// max_ne elements a block), else 0.  Eight blocks keep eight SMs busy where a launch per colour spreads the work, so the
+// elements a block may hold end where that costs more than the launches (eight overlapping ones take about 25 us back to
+// back).  Measured at 1 element to 256 threads a block, us with the cluster / with a launch per colour:
+//   FP64 element kernels, 128 threads (their FP64 pipe is the limit): p = 1, 256 elements 14 / 25; p = 2 Gauss, 64 elements
+//     20.6 / 25.1, 128 elements 28.8 / 25.2; p = 4, 40 elements 20.6 / 25.0, 80 elements 28.8 / 24.9; p = 8, 12 elements 43 / 31;
+//   FP32 and double-float, 256 threads: p = 3 FP32, 128 elements 16 / 24; p = 8 double-float, 24 elements 35 / 44;
+//   integer slices, one element: p = 7, 8 elements 20.8 / 24.5, 16 elements 26.7 / 24.4.
 constexpr int CLUSTER_BLOCKS = 8, CLUSTER_COLORS = 16;
+constexpr int cluster_max_elems(bool f64, bool slices, int Q) {
+  const int ne = (f64 ? 128 : 256) / (Q * Q);
+  return slices ? 1 : ne < 32 ? ne : 32;
+}
 inline int cluster_elems(int64_t E, int n_colors, int ncol, int max_ne) {
   if (ncol > CLUSTER_BLOCKS || n_colors > CLUSTER_COLORS) return 0;
   const int64_t per_column = CLUSTER_BLOCKS / ncol, ne = (E + per_column - 1) / per_column;

@@ -803,7 +803,7 @@ extern "C" int ceed_autotune_apply(ceed_mesh_t m, int op, const void *qdata, int
     return ms / reps;
   };
   const bool slices = prec == CEED_F64 && slice_operator(m->P, m->Q, op);
-  const int cluster = cluster_elems(m->E, m->n_colors, r.ncol, ne_max);
+  const int cluster = cluster_elems(m->E, m->n_colors, r.ncol, cluster_max_elems(prec == CEED_F64, slices, m->Q));
   if (slices || cluster > 0) {
     const float ms = time(-1, 1);
     if (ms > 0.f) {

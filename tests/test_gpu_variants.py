@@ -1,8 +1,8 @@
 """GPU test of the rule for the apply's launches: which variants a call runs, counted in a captured graph.
 
 A variant that is set launches one kernel per colour; the default runs a mesh that fits one cluster in one launch; an
-operator on the integer slices has no variants.  Boundaries of the cluster: 8 blocks of 256 threads, in the
-slice kernels 96 or 128 threads an element, so two elements a block and 16 in all.
+operator on the integer slices has no variants.  Boundaries of the cluster: 8 blocks of 128 threads in FP64, of 256 in
+the other precisions, of one element in the slice kernels.
 """
 import ctypes
 
@@ -79,10 +79,14 @@ def test_default_at_the_cluster_limit(p, qkind, op, prec):
     import paper_2109_05072_gb300 as ceed
     Q = p + 1 if qkind == "gll" else p + 2
     slices = prec == 0 and Q >= 6
-    full = 16 if slices else 8 * min(32, 256 // (Q * Q))
+    full = 8 if slices else 8 * min(32, (128 if prec == 0 else 256) // (Q * Q))
     for dims in ((full - 1, 1, 1), (full // 2, 2, 1), (full + 1, 1, 1), (full // 4, 2, 2)):
         m, mesh, qd, cop, f = _setup(ceed, p, qkind, op, prec, dims)
         x = torch.from_numpy(synthetic.uniform(m.n_ldof * 9, seed=4)).cuda()
+        x0 = x[: m.n_ldof].contiguous()
+        y0 = torch.empty_like(x0)
+        n = _launches(lambda: f(mesh, qd, prec, x0, y0))
+        assert n == (1 if m.n_elem <= full else mesh.n_colors)
         for flags in (0, ceed.CEED_APPLY_DIRICHLET):
             y = torch.full_like(x, float("nan"))
             f(mesh, qd, prec, x, y, 9, flags)
