@@ -127,6 +127,7 @@ inline int cluster_elems(int64_t E, int n_colors, int ncol, int max_ne) {
 // A value's eight balanced base-256 digits as FP16 bit patterns, leading digit first: the integer nearest
 // to v 2^scale, which has to lie below 2^62 (mesh.cu).
 void fix_digits_host(long double v, int scale, uint16_t *out);
+void fix_digits_host(double v, int scale, uint16_t *out);  // (no long double arithmetic, which Arm does in software)
 int fix_scale_host(const long double *M, size_t n);  // largest scale that keeps every entry below 2^62
 
 struct QRule {

@@ -216,8 +216,7 @@ int fix_scale_host(const long double *M, size_t n) {
   return 62 - ex;
 }
 
-void fix_digits_host(long double v, int scale, uint16_t *out) {
-  int64_t r = std::llrint(std::ldexp(v, scale));
+static void fix_digits_of(int64_t r, uint16_t *out) {
   for (int j = FIX_DIGITS - 1; j >= 0; --j) {
     const int dig = (int)(((r + 128) & 255) - 128);
     r = (r - dig) / 256;
@@ -225,6 +224,9 @@ void fix_digits_host(long double v, int scale, uint16_t *out) {
     std::memcpy(&out[j], &h, 2);
   }
 }
+
+void fix_digits_host(long double v, int scale, uint16_t *out) { fix_digits_of(std::llrint(std::ldexp(v, scale)), out); }
+void fix_digits_host(double v, int scale, uint16_t *out) { fix_digits_of(std::llrint(std::ldexp(v, scale)), out); }
 
 // Digit table of an NO x NI matrix (both at most 8) for the slice kernels' B fragments.  The matrix is the one that
 // the even-odd blocks stand for (symmetric or antisymmetric to the last bit), so that both kinds of kernel apply

@@ -325,20 +325,18 @@ __global__ void __launch_bounds__(32 * NTF_WARPS, ntf_blocks(NC)) nt_fix_kernel(
 // those in which a row has fewer than two entries within a factor of 16 of the table's largest (a nodal basis at its own
 // nodes): most elements would be computed twice.
 static bool nt_fix_scales(const double *M, int D, int Q, int P, int *fwd, int *bwd) {
-  std::vector<long double> big((size_t)D * Q * P);
-  long double most = 0, row = 0, col = 0;
-  for (size_t k = 0; k < big.size(); ++k) {
+  double most = 0, row = 0, col = 0;
+  for (size_t k = 0; k < (size_t)D * Q * P; ++k) {
     if (!std::isfinite(M[k])) return false;
-    big[k] = M[k];
-    most = std::max(most, std::fabs(big[k]));
+    most = std::max(most, std::fabs(M[k]));
   }
   if (most == 0) return false;
   for (int d = 0; d < D; ++d)
     for (int q = 0; q < Q; ++q) {
-      long double sum = 0;
+      double sum = 0;
       int large = 0;
       for (int n = 0; n < P; ++n) {
-        const long double v = std::fabs(big[((size_t)d * Q + q) * P + n]);
+        const double v = std::fabs(M[((size_t)d * Q + q) * P + n]);
         sum += v;
         large += v >= most / 16;
       }
@@ -347,17 +345,18 @@ static bool nt_fix_scales(const double *M, int D, int Q, int P, int *fwd, int *b
     }
   for (int q0 = 0; q0 < Q; q0 += 8)
     for (int n = 0; n < P; ++n) {
-      long double sum = 0;
+      double sum = 0;
       for (int d = 0; d < D; ++d)
-        for (int q = q0; q < std::min(Q, q0 + 8); ++q) sum += std::fabs(big[((size_t)d * Q + q) * P + n]);
+        for (int q = q0; q < std::min(Q, q0 + 8); ++q) sum += std::fabs(M[((size_t)d * Q + q) * P + n]);
       col = std::max(col, sum);
     }
-  int row_ex = 0, col_ex = 0;
-  std::frexp(row * 1.01L, &row_ex);
-  std::frexp(col * 1.01L, &col_ex);
-  const int scale = fix_scale_host(big.data(), big.size());
-  *fwd = std::min(scale, 66 - row_ex);
-  *bwd = std::min(scale, 66 - col_ex);
+  int most_ex = 0, row_ex = 0, col_ex = 0;
+  std::frexp(most, &most_ex);
+  std::frexp(row * 1.01, &row_ex);
+  std::frexp(col * 1.01, &col_ex);
+  if (!std::isfinite(row) || !std::isfinite(col)) return false;
+  *fwd = std::min(62 - most_ex, 66 - row_ex);
+  *bwd = std::min(62 - most_ex, 66 - col_ex);
   return std::min(*fwd, *bwd) >= 0 && std::max(*fwd, *bwd) <= 100;
 }
 
@@ -376,7 +375,8 @@ static int nt_fix_tables(ceed_nt_t h, const double *tab64, cudaStream_t s) {
         for (int n = 0; n < P; ++n) {
           uint16_t fd[FIX_DIGITS], bd[FIX_DIGITS];
           fix_digits_host(M[((size_t)d * Q + q) * P + n], scale[0], fd);
-          fix_digits_host(M[((size_t)d * Q + q) * P + n], scale[1], bd);
+          if (scale[1] == scale[0]) std::copy(fd, fd + FIX_DIGITS, bd);
+          else fix_digits_host(M[((size_t)d * Q + q) * P + n], scale[1], bd);
           const size_t tile = ((size_t)(q / 8) * D + d) * NC + n / 8;
           // forward: output point = lane / 4, input node pair = lane % 4; transposed: the other way round
           const size_t f = (tile * 32 + (q % 8) * 4 + (n % 8) / 2) * FIX_DIGITS;
