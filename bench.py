@@ -86,6 +86,18 @@ def algorithmic_bytes(m, qbytes, geo=False):
     return 16 * m.n_ldof + qd + 4 * m.n_elem * nd
 
 
+def fp64_pipe_flops(p, gauss=False):
+    """Flops per element (2 per instruction) that the FP64 diffusion operator leaves on the FP64 pipe.
+
+    Lines of 6 to 8 points (7 or 8 with Gauss quadrature) run their 1D passes as integer slices on the tensor cores:
+    the 3 x 3 product at a point (9 instructions) and the sum of the three directions (3) stay.  Other lines:
+    the paper's cost model (the even-odd operators execute about 0.8 of it)."""
+    q = p + 2 if gauss else p + 1
+    if (7 if gauss else 6) <= q <= 8:
+        return 24 * q ** 3
+    return 24 * (p + 1) ** 4 + 15 * q ** 3 if gauss else cost_per_element(p)[1]
+
+
 def load_peaks():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -310,7 +322,8 @@ def run_batched(ceed, dev, args, peaks=None, nrhs_list=(1, 4, 8, 16), steps=5, p
     out = {"meshes": [f"p={p}, {N}^3, Gauss q={p + 2}, n_ldof={n}" for (p, N), n in zip(specs, nodes)],
            "ncomp": 3, "dtype": "f64" if prec == ceed.CEED_F64 else "f32x2 (double-float, FP64-accurate)", "runs": [],
            "model": "per element and column 24 P^4 + 15 Q^3 flops (Section 2 model, contraction term doubled "
-                    "for q = p + 2); fp64_frac against the measured FP64 FMA rate"}
+                    "for q = p + 2); fp64_frac: what is left of that on the FP64 pipe (p = 5 runs its 1D passes on the "
+                    "tensor cores) against the measured FP64 FMA rate"}
     for nrhs in nrhs_list:
         xs = [torch.from_numpy(synthetic.uniform(n * 3 * nrhs, seed=7 + k)).to(dev) for k, n in enumerate(nodes)]
         ys = [torch.empty_like(x) for x in xs]
@@ -324,7 +337,8 @@ def run_batched(ceed, dev, args, peaks=None, nrhs_list=(1, 4, 8, 16), steps=5, p
         row = {"nrhs": nrhs, "ms_per_apply": ms, "gdofs": dofs / ms / 1e6, "threads": threads,
                "tma_staging": stage, "grid": grid, "launches_per_apply": 1, "model_tflops": flops / ms / 1e9}
         if peaks and peaks.get("f64") and prec == ceed.CEED_F64:
-            row["fp64_frac"] = row["model_tflops"] / peaks["f64"]["tflops"]
+            left = sum(fp64_pipe_flops(p, gauss=True) * N ** 3 for p, N in specs) * 3 * nrhs
+            row["fp64_frac"] = left / ms / 1e9 / peaks["f64"]["tflops"]
         out["runs"].append(row)
         batch.close()
         del xs, ys
@@ -671,10 +685,11 @@ def main():
     bytes64 = algorithmic_bytes(m, 8)
     launches_per_apply = mesh.n_colors
     v64 = variants.get("f64", {"elems_per_block": 1, "tma_staging": 0})
-    kernel_id = (f"apply_kernel<8,8,DIFFUSION,double,double,stage={v64['tma_staging']}>"
+    kernel_id = (f"fix_kernel<{p + 1},{p + 1},DIFFUSION>" if 5 <= p <= 7 else  # integer slices: one kernel, no variants
+                 f"apply_kernel<{p + 1},{p + 1},DIFFUSION,double,double,stage={v64['tma_staging']}>"
                  f"[ne={v64['elems_per_block']}]")
     ms_launch = ms64 / launches_per_apply
-    flops_launch = flops_el * m.n_elem / launches_per_apply
+    flops_launch = fp64_pipe_flops(p) * m.n_elem / launches_per_apply
     achieved_tf = flops_launch / (ms_launch * 1e-3) / 1e12
 
     # ---------------- FP64-accurate operator on the FP32 pipe (double-float), and its agreement with FP64
@@ -928,10 +943,11 @@ def main():
                          "peak_kind": "measured in this run: FP64 FMA chains on every SM (ceed_fma_throughput), "
                                       f"{peaks['f64']['sm_mhz']:.0f} MHz; nominal {FP64_NOMINAL_TFLOPS}",
                          "peak_nominal": FP64_NOMINAL_TFLOPS,
-                         "note": "achieved counts the paper's cost model (12 P^4 + 15 P^3 per element); the even-odd "
-                                 "1D operators execute about 0.8 of those flops, so frac reads above 1 while ncu "
-                                 "shows the FP64 pipe 85% busy",
+                         "note": "achieved counts what is left on the FP64 pipe: 12 instructions a point (pointwise step and "
+                                 "final sums, 2 flops each); the 1D passes run as exact integer slices on the tensor "
+                                 "cores.  model_tflops: the paper's cost model (12 P^4 + 15 P^3 per element)",
                          "flops_per_launch": flops_launch, "ms_per_launch": ms_launch,
+                         "model_tflops": flops_el * m.n_elem / (ms64 * 1e-3) / 1e12,
                          "hbm_gbs": bytes64 / (ms64 * 1e-3) / 1e9, "hbm_peak": hbm_peak, "hbm_peak_kind": hbm_kind,
                          "hbm_frac": bytes64 / (ms64 * 1e-3) / 1e9 / hbm_peak},
             "fp64_accurate_fp32_pipe": f64df,

@@ -26,6 +26,14 @@ def test_cost_model_and_algorithmic_bytes_of_the_headline():
     assert geo == 16 * m.n_ldof + (24 * 4 + 4 * 512) * m.n_elem + 4 * 512 * m.n_elem
 
 
+def test_work_left_on_the_fp64_pipe():
+    # lines of 6 to 8 points (Gauss: 7 or 8) leave 12 instructions a point; the others the cost model
+    assert bench.fp64_pipe_flops(7) == 24 * 512 and bench.fp64_pipe_flops(5) == 24 * 216
+    assert bench.fp64_pipe_flops(4) == bench.cost_per_element(4)[1] and bench.fp64_pipe_flops(8) == bench.cost_per_element(8)[1]
+    assert bench.fp64_pipe_flops(5, gauss=True) == 24 * 343
+    assert bench.fp64_pipe_flops(7, gauss=True) == 24 * 8 ** 4 + 15 * 9 ** 3
+
+
 def _fake_smi(tmp_path, startup_s, line):
     script = tmp_path / "nvidia-smi"
     script.write_text("#!%s\nimport sys, time\ntime.sleep(%r)\nwhile True:\n    print(%r, flush=True)\n"
