@@ -47,6 +47,11 @@ typedef enum {
 
 /* Precision of stored quadrature data; it also selects the operator arithmetic:
  * F64 -> FP64 contractions; F32/BF16/F16 -> FP32 contractions (FP64 L-vectors in and out).
+ * F64 with lines of 6 to 8 points (collocated diffusion; mass and diffusion with 7 or 8 Gauss points):
+ * a 1D contraction is formed on the tensor cores from exact integer slices, 62 bits below the line's
+ * largest value, and rounded once; relative to the sum of the magnitudes of an entry's terms it is as
+ * accurate as FP64 FMAs in the even-odd form that the other lines use.  Lines with values that are not
+ * finite, or whose largest is not zero and outside 2^-895 .. 2^877, take FP64 FMAs.
  * F32_GEO (diffusion only) -> FP32 contractions with the geometric factors recomputed from the
  * trilinear element map at every application: the quadrature data holds only the map's 8
  * coefficient vectors per element and w k per point (FP32), about 1/6 of the F32 bytes.
@@ -201,15 +206,15 @@ int ceed_manufactured_rhs(ceed_mesh_t mesh, int coeff_kind, double *b, unsigned 
 
 /* Several independent meshes -- polynomial orders may differ -- applied by ONE persistent kernel
  * launch (multi-right-hand-side batching and mixed order in one launch).  The launch is sized to the
- * thread blocks that are co-resident on the GPU; each block loops over the colours and over its share
- * of every mesh's elements of that colour, with a bounded grid-wide barrier between colours (the
- * atomic-free scatter needs colours in sequence).  The launch is captured once into a CUDA graph and
+ * thread blocks that are co-resident on the GPU; pieces of work (elements of one mesh and colour) are
+ * handed out in colour order, and a piece touches y once its mesh's colour before has been counted
+ * complete, behind a bounded wait (the atomic-free scatter needs colours in sequence).  The launch is captured once into a CUDA graph and
  * replayed by ceed_batch_apply.  Buffers are fixed at creation: qdata[k] (built for meshes[k] in
  * `prec`), x[k], y[k] (FP64, [n_ldof * ncomp * nrhs] of mesh k).  All meshes must use the same
  * quadrature rule kind (GLL or Gauss).  Supported: F64 and F64_DF (the FP64-accurate double-float
  * operator) mass/diffusion, F32 diffusion.  The batch must
  * not run concurrently with other kernels on the device (the persistent grid assumes it has the GPU);
- * if a barrier wait times out, ceed_batch_status returns CEED_ERR_TIMEOUT. */
+ * if a wait between colours times out, ceed_batch_status returns CEED_ERR_TIMEOUT. */
 typedef struct ceed_batch_s *ceed_batch_t;
 int ceed_batch_create(int n, const ceed_mesh_t *meshes, const void *const *qdata, int prec, int op,
                       const double *const *x, double *const *y, int nrhs, ceed_batch_t *out);
@@ -267,10 +272,11 @@ size_t ceed_cg_workspace_bytes(ceed_mesh_t mesh, const ceed_cg_opts *opts);
 /* Solve A x = b with Jacobi-preconditioned CG (Section 1) on the Dirichlet-masked operator.
  * Fused iteration (default where supported): one cooperative persistent kernel runs check_every
  * whole iterations -- the colour-ordered apply q = A p with p.q summed by each node's last writer,
- * alpha, x and r updates with the r.z and r.r sums (z = D^{-1} r is not stored), beta, p update --
- * separated by bounded grid barriers; reductions in a fixed order (results are reproducible run to
- * run, and differ from the separate-kernel path only in rounding order).  A barrier that gives up
- * returns CEED_ERR_TIMEOUT.
+ * alpha, x and r updates with the r.z and r.r sums (z = D^{-1} r stored for the p update), beta, p
+ * update.  Bounded grid barriers separate these steps, bounded waits on counters of finished work the
+ * colours of the apply; reductions in a fixed order (results are reproducible run to run, and differ
+ * from the separate-kernel path only in rounding order).  A wait that gives up returns
+ * CEED_ERR_TIMEOUT.
  * FP64 mode: all arithmetic FP64.  MIXED mode: iterative refinement, outer residual
  * r = b - A x with the FP64 operator (qdata, prec), inner PCG with the low-precision operator
  * (opts->qdata_lo, FP32 contractions, or the double-float operator of F64_DF) and FP64 vectors,
@@ -378,7 +384,12 @@ int ceed_apply_diffusion_adjoint(ceed_mesh_t mesh, const double *k, const void *
  * x(xi) = v0 + sum_d xi_d (v_d - v0) from 4 vertices (tetrahedra).  L-vectors are FP64 [n_ldof]
  * (one component).  Two algorithms, selectable per (op, prec):
  *   CEED_NT_FUSED  one fused kernel (gather, forward contraction, pointwise D, transposed
- *                  contraction in shared memory and registers), 32 elements per thread block;
+ *                  contraction in shared memory and registers), 32 elements per thread block.  F64
+ *                  with at most 35 basis functions: both contractions on the tensor cores as exact
+ *                  integer slices; an element in which a node's result would be less precise than by
+ *                  FP64 FMAs (values or table entries of very different size) is computed by them, and
+ *                  so are bases that do not suit the slices (a nodal basis at its own points, entries
+ *                  that are not finite or of extreme scale);
  *   CEED_NT_GEMM   the paper's GEMM formulation: the element inputs form one [E x P] matrix, each
  *                  basis action is one GEMM with the [P x D Q] basis matrix (cuBLAS), optionally
  *                  split into a strided batch of eta-element blocks; gemm_mode 0 = native
@@ -533,8 +544,8 @@ int ceed_mesh_status(ceed_mesh_t mesh, void *stream);
 /* Limits of the bounded device-side waits (not an operation of the paper; failure handling):
  * copy_polls governs each staging apply kernel's wait for its quadrature-data copy (negative: the default
  * bound of 2^22 polls; 0: give up at once; the kernels keep that bound a compile-time constant, so
- * other values are INVALID), barrier_polls the grid barriers of the persistent batched launch and of
- * the fused CG iteration (negative: the default 2^25 polls; 0 .. 2^25: that many polls).  A wait
+ * other values are INVALID), barrier_polls the waits between colours of the persistent batched launch
+ * and of the fused CG iteration and the latter's grid barriers (negative: the default 2^25 polls; 0 .. 2^25: that many polls).  A wait
  * that runs out records CEED_ERR_TIMEOUT (read by ceed_mesh_status / ceed_batch_status, returned by
  * ceed_cg_solve) and the kernel finishes without hanging; tests use 0 to drive these paths.
  * Process-wide; applies to launches issued afterwards (a batch's CUDA graph keeps the limits it was
