@@ -125,3 +125,30 @@ def test_copy_wait_expiry_of_the_colour_launches(prec):
     ceed.ceed_mesh_status(mesh)
     assert torch.equal(y, ref)
     mesh.close()
+
+
+@pytest.mark.parametrize("p,qkind,op,prec,dims", [(2, "gauss", "mass", 0, (4, 4, 4)), (7, "gll", "diffusion", 0, (4, 4, 3)),
+                                                  (3, "gll", "diffusion", 1, (8, 8, 6)), (3, "gll", "diffusion", 5, (8, 8, 6)),
+                                                  (6, "gauss", "diffusion", 0, (2, 2, 2))])
+def test_captured_applies_replay(p, qkind, op, prec, dims):
+    """Cluster and overlapping launches in a captured graph: every replay gives the bits of the call."""
+    import paper_2109_05072_gb300 as ceed
+    m, mesh, qd, cop, f = _setup(ceed, p, qkind, op, prec, dims)
+    x = torch.from_numpy(synthetic.uniform(m.n_ldof, seed=3)).cuda()
+    ref, y, z = torch.empty_like(x), torch.empty_like(x), torch.empty_like(x)
+    f(mesh, qd, prec, x, ref)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        f(mesh, qd, prec, x, y)
+        f(mesh, qd, prec, y, z)
+    for _ in range(3):
+        y.fill_(float("nan"))
+        z.fill_(float("nan"))
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, ref)
+        zz = torch.empty_like(x)
+        f(mesh, qd, prec, y, zz)
+        assert torch.equal(z, zz)
+    mesh.close()
