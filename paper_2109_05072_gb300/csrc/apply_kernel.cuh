@@ -140,16 +140,25 @@ __device__ __forceinline__ bool mbar_wait_n(uint64_t *bar, uint32_t parity, int 
 // 64,000 at p = 7 in FP32 445 -> 386 us.
 __device__ __forceinline__ void colour_open_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 struct ColourWait {
+  static constexpr bool OPEN = false;
   __device__ __forceinline__ bool operator()() const {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return true;
   }
+};
+// The first colour waits for nothing (it is launched as any kernel), so its y is open from the start.  A kernel of its own
+// for the FP32 pipe: where y may be read only behind the wait the compiler's schedule is slower, which shows where nothing
+// overlaps, on meshes of one colour (9,216 separate elements with 9 Gauss points: 95 us, 65 so; 6,912 at p = 8: 72, 52).
+struct ColourFirst {
+  static constexpr bool OPEN = true;
+  __device__ __forceinline__ bool operator()() const { return true; }
 };
 
 // A mesh small enough for one thread-block cluster: all its colours in one launch.  Every block gathers and
 // computes its elements at once, then the colours take turns at y, a cluster barrier between them (y is
 // read and written through L2).
 struct ClusterOrder {
+  static constexpr bool OPEN = false;
   int ncolors;
   int start[CLUSTER_COLORS + 1];   // colour-sorted element ranges
   // f(true) in element e's turn, f(false) in the others
@@ -608,8 +617,9 @@ inline void column_split(ApplyArgs &a, int64_t eblocks) {
 // XCG: x is read through L2 only (ld.global.cg) instead of the read-only path: required when x
 // changes during the kernel (the persistent CG iteration updates p between its applies).
 // SPLIT: false if a block does all columns of its elements (a.cgroups = 1).  A path of its own for the double-float
-// kernels, which run at their register cap: with the group's arithmetic in the way 64^3 at p = 7 took 3.42 ms, and
-// 24^3 at p = 8 0.585 (one column) and 2.46 ms (four), against 3.06, 0.517 and 2.13 without; the others gain nothing.
+// kernels, which run at their register cap (with the group's arithmetic in the way 64^3 at p = 7 took 3.42 ms, and
+// 24^3 at p = 8 0.585 (one column) and 2.46 ms (four), against 3.06, 0.517 and 2.13 without), and for the FP32 pipe
+// (24^3, p = 7, geometry on the fly: 96 against 75 us; others 1 to 2%).  The FP64 kernels gain nothing.
 // wait_y: called by every thread of the block before its first access to y (earlier colours written);
 // false if it gave up, and the block then writes nothing.
 template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool XCG = false, bool SPLIT = !XCG, typename WaitY>
@@ -680,8 +690,8 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
 
   for (int col = col0; col < col1; ++col) {
     // ---- x at my nodes, every load of the column up front; the old y where an earlier colour wrote
-    // with them from the second column on (the first loads it at the scatter, behind the earlier
-    // colours' writes; the double-float operator always does, as holding it across the element would
+    // with them from the second column on, or where y is open (else the first column loads it at the scatter, behind the
+    // earlier colours' writes; the double-float operator always does, as holding it across the element would
     // cost 2P registers of occupancy)
     constexpr bool EARLY_YOLD = !std::is_same<T, DF>::value;
     double xv[P], yold[P];
@@ -694,7 +704,7 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
         const int64_t o = (int64_t)(v & DOF_MASK) * a.ncol + col;
         const bool dir = a.masked && (v & FLAG_DIR);
         if (!dir) xv[c] = XCG ? __ldcg(a.x + o) : __ldg(a.x + o);
-        if (EARLY_YOLD && col > col0 && y_ok && !dir && !(v & FLAG_FIRST)) yold[c] = __ldcg(a.y + o);
+        if (EARLY_YOLD && (WaitY::OPEN || col > col0) && y_ok && !dir && !(v & FLAG_FIRST)) yold[c] = __ldcg(a.y + o);
       }
     }
     T u[P];
@@ -731,7 +741,7 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
       y_ok = wait_y();
     }
     const bool fused_dot = a.dot_part || a.dot_sh;
-    if (!EARLY_YOLD || col == col0) {
+    if (!EARLY_YOLD || (!WaitY::OPEN && col == col0)) {
 #pragma unroll
       for (int c = 0; c < P; ++c) {
         if (active && node_thread && q_ok && y_ok) {
@@ -802,14 +812,14 @@ __device__ __forceinline__ void apply_block(const ApplyArgs &a, const OpTab<T> &
   }
 }
 
-template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
+template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool SPLIT, bool FIRST>
 __global__ void __launch_bounds__(APPLY_MAX_THREADS)
 apply_kernel(const ApplyArgs a, const OpTab<T> tab) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bar[STAGE ? APPLY_MAX_NE : 1];
-  ColourWait wait_y;
+  const std::conditional_t<FIRST, ColourFirst, ColourWait> wait_y{};
   colour_open_next();
-  apply_block<P, Q, OP, T, TQ, STAGE>(a, tab, blockIdx.x, smem_raw, bar, wait_y);
+  apply_block<P, Q, OP, T, TQ, STAGE, false, SPLIT>(a, tab, blockIdx.x, smem_raw, bar, wait_y);
 }
 
 // The double-float instantiations under a register cap: that operator is bound by latency
@@ -896,12 +906,17 @@ template <int P, int Q, int OP, typename T, typename TQ, bool STAGE>
 int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne, bool by_default, cudaStream_t s) {
   const size_t smem = (size_t)ne * apply_elem_smem<P, Q, OP, T, TQ, STAGE>();
   constexpr bool CAPPED = std::is_same<T, DF>::value;
-  if constexpr (CAPPED) {
-    if (int st = ensure_dynamic_smem((const void *)apply_kernel_capped<P, Q, OP, T, TQ, STAGE, false>, smem)) return st;
-    if (int st = ensure_dynamic_smem((const void *)apply_kernel_capped<P, Q, OP, T, TQ, STAGE, true>, smem)) return st;
-  } else {
-    if (int st = ensure_dynamic_smem((const void *)apply_kernel<P, Q, OP, T, TQ, STAGE>, smem)) return st;
-  }
+  constexpr bool FP32 = std::is_same<T, float>::value;
+  const auto kernel_of = [](auto split, auto first) {
+    if constexpr (CAPPED) return apply_kernel_capped<P, Q, OP, T, TQ, STAGE, decltype(split)::value>;
+    else return apply_kernel<P, Q, OP, T, TQ, STAGE, decltype(split)::value, decltype(first)::value>;
+  };
+  const auto split_kernel = kernel_of(std::true_type(), std::false_type());
+  const auto whole_kernel = kernel_of(std::bool_constant<!CAPPED && !FP32>(), std::false_type());  // (FP64: one for both)
+  const auto first_kernel = kernel_of(std::bool_constant<!CAPPED && !FP32>(), std::bool_constant<FP32>());
+  if (int st = ensure_dynamic_smem((const void *)split_kernel, smem)) return st;
+  if (int st = ensure_dynamic_smem((const void *)whole_kernel, smem)) return st;
+  if (int st = ensure_dynamic_smem((const void *)first_kernel, smem)) return st;
   const dim3 block(Q * Q * ne);
   ApplyArgs a;
   a.emap = m->d_emap;
@@ -936,11 +951,7 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
     a.e_count = n;
     column_split(a, (n + ne - 1) / ne);
     const dim3 grid((unsigned)((n + ne - 1) / ne * a.cgroups));
-    int st;
-    if constexpr (CAPPED)
-      st = launch_colour(a.cgroups > 1 ? apply_kernel_capped<P, Q, OP, T, TQ, STAGE, true> : apply_kernel_capped<P, Q, OP, T, TQ, STAGE, false>,
-                         grid, block, smem, s, first, a, tab);
-    else st = launch_colour(apply_kernel<P, Q, OP, T, TQ, STAGE>, grid, block, smem, s, first, a, tab);
+    const int st = launch_colour(a.cgroups > 1 ? split_kernel : first ? first_kernel : whole_kernel, grid, block, smem, s, first, a, tab);
     if (st) return st;
     first = false;
     a.dot_base += grid.x;

@@ -88,6 +88,7 @@ __device__ __forceinline__ int64_t pieces(const BatchArgs<T> &b, int c, int m) {
 // piece never waits, and all that a piece does before its scatter (gather, contractions) overlaps the
 // colour before.  The wait is bounded like the grid barrier's.
 struct ColourOrder {
+  static constexpr bool OPEN = false;
   const unsigned *prev;   // counter of the colour before; null: nothing to wait for, or waited for already
   unsigned target;
   long long limit;
