@@ -209,8 +209,8 @@ __device__ __forceinline__ void cg_fused_body(const CgFusedArgs &g, const OpTab<
   }
 }
 
-// register caps of the fused iteration (measured at 64^3, p = 7 on the GB300 against the separate
-// kernels, ms per iteration: FP32 operator 3.18 vs 3.47, FP64 14.81 vs 14.73 (uncapped: 15.9))
+// register caps of the fused iteration (64^3, p = 7, ms per iteration against the separate kernels: FP32 operator 3.33
+// vs 3.60, double-float 5.99 vs 7.38, FP64 on the integer slices 7.97 vs 7.54; FP64 element kernels, p = 3, 1.49 vs 1.43)
 #ifndef CGF_F32_MAX_REGS
 #define CGF_F32_MAX_REGS 96
 #endif

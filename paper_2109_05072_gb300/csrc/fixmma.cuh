@@ -85,7 +85,7 @@ constexpr uint32_t FIX_MAGIC = 0x4B400000u;  // bits of 1.5 * 2^23: bits(magic +
 
 // Eight orders (bit patterns of magic + sum) to FP64: sum_s u_s 2^(47 - 8 s), rounded once; eb is the
 // exponent field of the sum's unit plus 62.  The sum stays below 2^63 if the table's entries of one product sum
-// to less than 2^65 (eight entries always do).  Orders 6 and 7 are rounded to whole units, without bias
+// to less than 2^66 (eight entries always do).  Orders 6 and 7 are rounded to whole units, without bias
 // and a zero to zero.
 __device__ __forceinline__ double fix_out(const uint32_t (&u)[FIX_DIGITS], int eb) {
   constexpr uint64_t K = (uint64_t)FIX_MAGIC * ((1ull << 47) + (1ull << 39) + (1ull << 31) + (1ull << 23) + (1ull << 15) + (1ull << 7)) +

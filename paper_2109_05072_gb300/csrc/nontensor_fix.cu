@@ -38,8 +38,8 @@ namespace ceedgb {
 
 constexpr int NTF_WARPS = 4;
 // Blocks per SM by node chunks: the warps of a group's chain of passes wait on one another's results most of the time, so
-// more of them pay for some spilled registers (degree 4: 1.55 ms with two blocks, 1.19 with three, 1.26 with four;
-// degrees 1 to 3: 0.47, 0.68, 0.78 ms with three, 0.41, 0.54, 0.67 with four).
+// more of them pay for some spilled registers (diffusion of degree 4: 1.58 ms with two blocks, 1.09 with three, 1.21 with four;
+// degrees 1 to 3: 0.57, 0.65, 0.76 ms with three, 0.49, 0.59, 0.69 with four).
 constexpr int ntf_blocks(int nc) { return nc > 4 ? 3 : 4; }
 
 bool nt_fix_supported(ceed_nt_t h, int op) { return h->d_fix[op == CEED_OP_MASS ? 0 : 1] != nullptr; }
