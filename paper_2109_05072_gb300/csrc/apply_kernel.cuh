@@ -146,9 +146,10 @@ struct ColourWait {
     return true;
   }
 };
-// The first colour waits for nothing (it is launched as any kernel), so its y is open from the start.  A kernel of its own
-// for the FP32 pipe: where y may be read only behind the wait the compiler's schedule is slower, which shows where nothing
-// overlaps, on meshes of one colour (9,216 separate elements with 9 Gauss points: 95 us, 65 so; 6,912 at p = 8: 72, 52).
+// The only colour of a mesh waits for nothing, so its y is open from the start.  A kernel of its own for the FP32 pipe: where
+// y may be read only behind the wait the compiler's schedule is slower, which shows where nothing overlaps (9,216
+// separate elements with 9 Gauss points: 95 us, 65 so; 6,912 at p = 8: 72, 52).  Not for the first of several: 64^3 at
+// p = 7 with BF16 data took 1.18 ms with one kernel for all colours, 1.46 with another for the first.
 struct ColourFirst {
   static constexpr bool OPEN = true;
   __device__ __forceinline__ bool operator()() const { return true; }
@@ -618,8 +619,9 @@ inline void column_split(ApplyArgs &a, int64_t eblocks) {
 // changes during the kernel (the persistent CG iteration updates p between its applies).
 // SPLIT: false if a block does all columns of its elements (a.cgroups = 1).  A path of its own for the double-float
 // kernels, which run at their register cap (with the group's arithmetic in the way 64^3 at p = 7 took 3.42 ms, and
-// 24^3 at p = 8 0.585 (one column) and 2.46 ms (four), against 3.06, 0.517 and 2.13 without), and for the FP32 pipe
-// (24^3, p = 7, geometry on the fly: 96 against 75 us; others 1 to 2%).  The FP64 kernels gain nothing.
+// 24^3 at p = 8 0.585 (one column) and 2.46 ms (four), against 3.06, 0.517 and 2.13 without), and for FP32 with geometry on
+// the fly (24^3, p = 7, staged: 96 against 79 us).  The FP64 kernels gain nothing, FP32 3% either way, and BF16 data
+// loses (24^3, p = 7, staged, two elements a block: 67 against 73 us).
 // wait_y: called by every thread of the block before its first access to y (earlier colours written);
 // false if it gave up, and the block then writes nothing.
 template <int P, int Q, int OP, typename T, typename TQ, bool STAGE, bool XCG = false, bool SPLIT = !XCG, typename WaitY>
@@ -912,7 +914,8 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
     else return apply_kernel<P, Q, OP, T, TQ, STAGE, decltype(split)::value, decltype(first)::value>;
   };
   const auto split_kernel = kernel_of(std::true_type(), std::false_type());
-  const auto whole_kernel = kernel_of(std::bool_constant<!CAPPED && !FP32>(), std::false_type());  // (FP64: one for both)
+  constexpr bool WHOLE = CAPPED || OP == OP_DIFF_GEO;
+  const auto whole_kernel = kernel_of(std::bool_constant<!WHOLE>(), std::false_type());  // (else one for both)
   const auto first_kernel = kernel_of(std::bool_constant<!CAPPED && !FP32>(), std::bool_constant<FP32>());
   if (int st = ensure_dynamic_smem((const void *)split_kernel, smem)) return st;
   if (int st = ensure_dynamic_smem((const void *)whole_kernel, smem)) return st;
@@ -951,7 +954,7 @@ int launch_variant(ceed_mesh_t m, const OpTab<T> &tab, const ApplyReq &r, int ne
     a.e_count = n;
     column_split(a, (n + ne - 1) / ne);
     const dim3 grid((unsigned)((n + ne - 1) / ne * a.cgroups));
-    const int st = launch_colour(a.cgroups > 1 ? split_kernel : first ? first_kernel : whole_kernel, grid, block, smem, s, first, a, tab);
+    const int st = launch_colour(a.cgroups > 1 ? split_kernel : m->n_colors == 1 ? first_kernel : whole_kernel, grid, block, smem, s, first, a, tab);
     if (st) return st;
     first = false;
     a.dot_base += grid.x;
